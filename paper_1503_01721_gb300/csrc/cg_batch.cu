@@ -291,6 +291,7 @@ static vmat_status make_batch(Batch &b, int32_t n_plans, const vmat_plan_desc *p
         VMAT_TRY(b.get((char **)&p.obj_ws, objective_scratch_bytes(ctx->n_sm)));
         VMAT_TRY(b.get((char **)&p.pr_ws, pricing_scratch_bytes(&p.mlc)));
         VMAT_TRY(b.get((char **)&p.mp_ws, mp_workspace_bytes(std::min(nap, 96))));
+        VMAT_TRY(mp_workspace_clear(p.mp_ws, std::min(nap, 96), s));
         VMAT_TRY(b.get(&cpo_dev[i], (size_t)p.K + 1));
         VMAT_TRY(b.get(&p.win, (size_t)p.K * p.NR));
         VMAT_TRY(b.get(&p.live_flag, (size_t)p.n_wtiles));

@@ -329,6 +329,7 @@ extern "C" vmat_status cg_plan(vmat_ddc hd, const vmat_mlc *mlc, const vmat_voxe
     const int n_cap = std::min(std::max(n_apertures, 1), 96);
     void *mp_ws;
     VMAT_TRY(ar.get((char **)&mp_ws, mp_workspace_bytes(n_cap)));
+    VMAT_TRY(mp_workspace_clear(mp_ws, n_cap, s));
     double *mp_bytes_dev; // bytes the persistent master-problem passes moved
     VMAT_TRY(ar.get(&mp_bytes_dev, 1));
     VMAT_CUDA(cudaMemsetAsync(mp_bytes_dev, 0, sizeof(double), s));

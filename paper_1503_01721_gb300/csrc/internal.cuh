@@ -421,8 +421,10 @@ struct BBWork; // defined in mp_bb.cu
 int64_t mp_wtile_stride(int32_t n_cap);
 vmat_status mp_write_labels(const uint8_t *sid, int32_t V, int64_t wstride, float *DA, cudaStream_t s);
 // Device-driven solve (persistent solver only, n_ap <= n_cap <= 96): no host synchronisation;
-// ws holds mp_workspace_bytes(n_cap) bytes; skip and iters_acc as in the solver's arguments.
+// ws holds mp_workspace_bytes(n_cap) bytes, cleared (mp_workspace_clear) before its first solve
+// and kept as it is from solve to solve; skip and iters_acc as in the solver's arguments.
 size_t mp_workspace_bytes(int32_t n_cap);
+vmat_status mp_workspace_clear(void *ws, int32_t n_cap, cudaStream_t s);
 // Live warp tiles of a plan's master problem.  A voxel that no placed aperture
 // reaches has an all-zero row of DA: its dose is 0 whatever y is, and its penalty a
 // constant (Eq. 1 at z = 0).  The solver runs over the 32-voxel tiles that some

@@ -20,10 +20,11 @@
 // per iteration.  Objective terms w d^2 are formed in FP32 and summed per lane
 // with compensation (Kahan), then as float pairs across lanes and CTAs: the
 // voxel loop runs no FP64 instruction (FP64 issues at a small fraction of the
-// FP32 rate on this GPU).  After a grid barrier one warp per column reduces the
-// CTA partials in a fixed order; after a second barrier every CTA takes the
-// same step in shared memory: the Eq. 9-10 freeze, the stopping tests, the BB
-// step length (FP64) and the projected update.  The first iteration's Cauchy
+// FP32 rate on this GPU).  The CTA partials of every column are then summed in a
+// fixed order by one CTA each and the sums sent to all (exchange_columns: tagged
+// words, no barrier), and every CTA takes the same step in shared memory: the
+// Eq. 9-10 freeze, the stopping tests, the BB step length (FP64) and the projected
+// update.  The first iteration's Cauchy
 // step needs DA G and one more pass.
 //
 // Readings (where the paper is silent): G is the gradient of F, so both BB
@@ -47,6 +48,7 @@ constexpr int MP_WT = 32;       // voxels per warp tile
 constexpr int MP_HEAD = 32;     // floats of a warp tile's label head (128 bytes)
 constexpr int MP_CHUNK = 8;     // iterations launched between host polls
 constexpr size_t MP_SMEM_LIMIT = 220 * 1024;
+constexpr int RES_COPIES = 32; // copies of the reduced columns (a lane of the owner's warp writes each)
 constexpr int MP_NMAX = 96; // register-resident gradient shares: up to 96 apertures
 
 struct BBState {
@@ -75,16 +77,18 @@ struct MPArgs {
     const float *lo, *hi; // may be null
     double *G, *Gprev;
     float *yprev;
-    double *part;  // fallback solver: [P][n + 1] doubles; persistent solver: two buffers (by iteration
-                   // parity) of float pairs, [2][n + 1][pstride] (column k of CTA c at k * pstride + c)
-    double *cpart; // [P]
+    double *part;  // fallback solver: [P][n + 1] doubles
+    double *cpart; // fallback solver: [P]
     int32_t P;
-    int32_t pstride; // CTAs a persistent partial buffer has room for
+    // exchange of the persistent solvers (see exchange_columns): tagged float pairs
+    ulonglong2 *slots; // [n + 1][pstride]: column k of CTA c at k * pstride + c
+    ulonglong2 *res;   // [RES_COPIES][rstride]: the reduced columns, then the elastic solver's epoch
+    int32_t rstride;
+    unsigned *tag;     // tags up to this one have been used in slots and res
+    int32_t pstride;   // CTAs a column of slots has room for
     int32_t n_tiles;  // 256-voxel tiles (fallback and Cauchy kernels)
     int64_t n_wtiles; // 32-voxel warp tiles
     BBState *st;
-    unsigned *bar_count, *bar_gen; // grid barrier of the persistent solver
-    unsigned *epoch_snap;          // elastic batched solver: the batch epoch seen at this problem's last barrier
     const int32_t *skip;           // when non-null and set, the solve is skipped (device-driven plans)
     int32_t *iters_acc;            // when non-null, the persistent solver adds its iteration count
     double *bytes_acc;             // when non-null, the persistent solver adds the bytes its passes moved
@@ -103,6 +107,13 @@ struct MPArgs {
     const int32_t *poff;
 };
 
+// A value that is the same in the whole warp, in a form the compiler knows to be so: branches
+// and loops on it are then uniform.  Inside a branch on threadIdx.x / 32, or a loop to a
+// bound read from shared memory, it cannot rule out a diverged warp, and every shuffle and
+// vote there took 230 cycles instead of 31.
+__device__ __forceinline__ int warp_uniform(int x) { return __shfl_sync(0xffffffffu, x, 0); }
+__device__ __forceinline__ int warp_index() { return warp_uniform((int)(threadIdx.x >> 5)); }
+
 __device__ __forceinline__ int64_t min64(int64_t x, int64_t y) { return x < y ? x : y; }
 
 // Offset of DA(voxel i, aperture k) in the warp-tile layout.
@@ -119,10 +130,6 @@ __global__ void mp_init_kernel(MPArgs a) {
     if (threadIdx.x == 0) {
         BBState s = {};
         *a.st = s;
-        if (a.bar_count) {
-            *a.bar_count = 0u;
-            *a.bar_gen = 0u;
-        }
     }
 }
 
@@ -310,9 +317,8 @@ __host__ __device__ constexpr size_t wt_copy_bytes(int n) { return 128 + (size_t
 
 // ---------------------------------------------------------------------------
 // Persistent solver: one cooperative launch runs the whole BB loop.  Every
-// iteration is a pass over DA (each warp streams its own tiles), a grid
-// barrier, a column reduction of the CTA partials (one warp per column), a
-// second grid barrier, and the step, which every CTA computes identically in
+// iteration is a pass over DA (each warp streams its own tiles), the exchange of
+// the CTA partials' sums, and the step, which every CTA computes identically in
 // its own shared memory from the same reduced values.  Cross-thread sums of
 // FP32 values are formed as unevaluated float pairs (hi + lo, Knuth's TwoSum),
 // in a fixed order; the BB dot products, F and the step stay FP64.
@@ -336,72 +342,112 @@ __device__ __forceinline__ FF ff_shfl_xor(FF v, int d) {
     return FF{__shfl_xor_sync(0xffffffffu, v.hi, d), __shfl_xor_sync(0xffffffffu, v.lo, d)};
 }
 
+// The warp's sum of one float pair per lane (fixed butterfly, every lane).
+__device__ __forceinline__ FF warp_ff(FF v) {
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) v = ff_add(v, ff_shfl_xor(v, d));
+    return v;
+}
 __device__ __forceinline__ double ff_to_double(FF v) { return (double)v.hi + (double)v.lo; }
 
-// Grid barrier over n_cta co-resident CTAs (cooperative launch): arrival counter
-// plus a generation word.  Gives up after WAIT_LIMIT_CYCLES; returns false then.
-// When snap_dst is given, the last CTA to arrive copies *snap_src there before it
-// releases the others, so every CTA of the barrier reads the same value after it.
-__device__ bool grid_sync(unsigned *count, unsigned *gen, unsigned n_cta, unsigned *snap_dst = nullptr,
-                          const unsigned *snap_src = nullptr) {
-    __shared__ int ok_s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        volatile unsigned *vg = gen;
-        const unsigned g0 = *vg;
-        __threadfence();
-        int ok = 1;
-        if (atomicAdd(count, 1u) == n_cta - 1) {
-            if (snap_dst) *(volatile unsigned *)snap_dst = *(const volatile unsigned *)snap_src;
-            atomicExch(count, 0u);
-            __threadfence();
-            atomicAdd(gen, 1u);
-        } else {
-            const long long t0 = clock64();
-            while (*vg == g0) {
-                if (clock64() - t0 > WAIT_LIMIT_CYCLES) {
-                    ok = 0;
-                    break;
-                }
-                __nanosleep(64);
+// ---------------------------------------------------------------------------
+// Column sums over the CTAs of a solve, and their broadcast, without a grid barrier.
+//
+// A float pair travels as two 64-bit words, each (float bits, tag): a reader polls the
+// words until both carry the tag of the current exchange, so a value and the news of its
+// arrival are one access, with no fence, counter or barrier between writer and reader.
+// The results are written RES_COPIES times (one per lane of the owner's warp), each copy
+// polled by a share of the CTAs: with one copy the polls of 600 CTAs on one or two lines
+// held up the stores they waited for.
+// Every CTA writes its partial of column k to slot (k, cta); the CTA that owns column k
+// (CTA k, or with fewer CTAs than columns a warp of CTA k mod CTAs) polls the column's
+// slots, sums them in a fixed order and writes res[k]; every CTA polls res.  One buffer
+// is enough: a CTA writes a slot of exchange e + 1 only after it has read every result of
+// exchange e, whose owners had then read every slot of e; and an owner writes res[k] of
+// e + 1 only after every CTA's partial of e + 1, sent after that CTA had read res of e.
+// Tags grow by one per exchange over all solves on a workspace (zeroed when allocated);
+// CTAs of a solve are never more than one exchange apart.
+//
+// What bounds it: two trips through L2 (a store is seen by another SM's poll after about
+// 500 cycles on the same die, 870 on the other one), an owner's chain of additions and the
+// wait for the slowest CTA.  Measured per iteration (cycles, exchange and step; before: a
+// grid barrier, every CTA reducing every column, and the step): 40^3 voxels, 16
+// apertures, 250 CTAs: 10.5K -> 9.7K; 422K voxels, 40 apertures, 304 CTAs: 19.7K -> 12.1K;
+// 1.1M voxels, 56 apertures, 152 CTAs: 13.7K -> 10.3K.  That master problem (422K voxels, 40
+// apertures, 185 iterations) takes 3.24 ms instead of 4.16 ms, the 40^3 plan of 20
+// apertures 9.14 ms instead of 10.29 ms.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void tagged_store(ulonglong2 *p, FF v, unsigned tag) {
+    const unsigned long long hi = ((unsigned long long)tag << 32) | __float_as_uint(v.hi);
+    const unsigned long long lo = ((unsigned long long)tag << 32) | __float_as_uint(v.lo);
+    asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"(hi), "l"(lo) : "memory");
+}
+__device__ __forceinline__ ulonglong2 tagged_load(const ulonglong2 *p) {
+    ulonglong2 v;
+    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ bool tagged_ok(ulonglong2 v, unsigned tag) {
+    return (unsigned)(v.x >> 32) == tag && (unsigned)(v.y >> 32) == tag;
+}
+__device__ __forceinline__ FF tagged_value(ulonglong2 v) {
+    return FF{__uint_as_float((unsigned)v.x), __uint_as_float((unsigned)v.y)};
+}
+// The sum of one column's slots by a warp: lane l adds CTAs l, l + 32, ... in order, then a
+// fixed butterfly (the result in every lane).  SLOT_BATCH slots per lane are polled
+// together (few: more loads in flight here cost the solver's pass its registers).
+// Returns false when a slot never arrived.
+constexpr int SLOT_BATCH = 2;
+__device__ __forceinline__ bool column_sum(const ulonglong2 *col, int n_cta, unsigned tag, FF *out) {
+    const int lane = threadIdx.x & 31;
+    FF v{0.f, 0.f};
+    const long long t0 = clock64();
+    for (int b0 = 0; b0 < n_cta; b0 += 32 * SLOT_BATCH) { // warp-uniform
+        ulonglong2 q[SLOT_BATCH];
+        while (true) {
+            bool good = true;
+#pragma unroll
+            for (int u = 0; u < SLOT_BATCH; ++u) {
+                const int b = b0 + 32 * u + lane;
+                if (b < n_cta) q[u] = tagged_load(col + b);
             }
+#pragma unroll
+            for (int u = 0; u < SLOT_BATCH; ++u)
+                if (b0 + 32 * u + lane < n_cta) good = good && tagged_ok(q[u], tag);
+            if (__all_sync(0xffffffffu, good)) break;
+            if (__any_sync(0xffffffffu, clock64() - t0 > WAIT_LIMIT_CYCLES)) return false;
         }
-        __threadfence();
-        ok_s = ok;
+#pragma unroll
+        for (int u = 0; u < SLOT_BATCH; ++u)
+            if (b0 + 32 * u + lane < n_cta) v = ff_add(v, tagged_value(q[u]));
     }
-    __syncthreads();
-    return ok_s != 0;
+    *out = warp_ff(v);
+    return true;
 }
 
-// Grid barrier of a solve whose CTAs stay with it from start to end: one arrival
-// counter that only grows (zeroed by the init kernel before the launch); the e-th
-// barrier (e = 1, 2, ...) ends when the counter reaches e n_cta.  No CTA reads a word
-// before it arrives and no CTA resets one after the last arrival, so the barrier ends
-// one round trip after the last arrival.  Gives up after WAIT_LIMIT_CYCLES; returns
-// false then.
-__device__ bool grid_sync_count(unsigned *count, unsigned target) {
-    __shared__ int ok_c;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        atomicAdd(count, 1u);
-        int ok = 1;
-        const long long t0 = clock64();
-        while (true) {
-            unsigned v;
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(count) : "memory");
-            if ((int)(v - target) >= 0) break;
-            if (clock64() - t0 > WAIT_LIMIT_CYCLES) {
-                ok = 0;
-                break;
-            }
-            __nanosleep(32);
+// The same sum by the whole CTA: every thread polls the slots tid, tid + 256, ... and
+// stages their pairs, then the last warp adds them in the order above (the result in its
+// lanes).  stage: room for n_cta pairs.  Returns false, in every thread, when a slot never
+// arrived.
+__device__ __forceinline__ bool column_sum_cta(const ulonglong2 *col, int n_cta, unsigned tag, FF *stage, int wid,
+                                               FF *out) {
+    bool ok = true;
+    const long long t0 = clock64();
+    for (int b = threadIdx.x; b < n_cta && ok; b += MP_THREADS) {
+        ulonglong2 w = tagged_load(col + b);
+        while (ok && !tagged_ok(w, tag)) {
+            ok = clock64() - t0 <= WAIT_LIMIT_CYCLES;
+            w = tagged_load(col + b);
         }
-        __threadfence();
-        ok_c = ok;
+        stage[b] = tagged_value(w);
     }
-    __syncthreads();
-    return ok_c != 0;
+    if (!__syncthreads_and(ok)) return false;
+    if (wid == MP_NW - 1) {
+        FF v{0.f, 0.f};
+        for (int b = threadIdx.x & 31; b < n_cta; b += 32) v = ff_add(v, stage[b]);
+        *out = warp_ff(v);
+    }
+    return true;
 }
 
 // Barrier of the whole batched grid.  The last CTA to arrive records the batch
@@ -411,35 +457,58 @@ __device__ bool grid_sync_count(unsigned *count, unsigned target) {
 struct MPArgs;
 __device__ bool batch_sync(unsigned *gctl, unsigned n_cta, const MPArgs *args, int n_plans);
 
-// Solver state every CTA keeps in shared memory (identical in all CTAs).
+// Solver state every CTA keeps in shared memory (identical in all CTAs but for cta), and
+// what the end of an iteration needs of the solve's arguments.
 struct PState {
     double F_hist[6];
     double F, delta0, gg, delta;
-    int t, done, stop, decided;
-    int passes; // passes over DA (iterations and the Cauchy pass)
+    double F_off; // the constant of the tiles not in the solve (*F_off_dev)
+    int t, done, stop;
+    unsigned tag;   // of the last exchange
+    unsigned epoch; // elastic solver: the batch epoch the last exchange brought
+    int passes;     // passes over DA (iterations and the Cauchy pass)
     int stop_rel, stop_step; // the step's stopping tests, formed in parallel
-    double delta_c;          // the step's BB step size, formed in parallel
+    int abort;      // a wait of this CTA ran out
+    // set by solve_begin
+    int n, nmax, off; // apertures, their rounded count, byte offset of the arrays in dynamic shared memory
+    unsigned cta, n_cta;
+    ulonglong2 *slots, *res;
+    int pstride, rstride;
+    const unsigned *epoch_src;
+    const float *lo, *hi;
+    vmat_bb_opts opts;
+    double F_offset;
 };
+// One object per CTA: every function that names it gets the same shared variable.
+__device__ __forceinline__ PState &solve_state() {
+    __shared__ PState ps;
+    return ps;
+}
 
 struct SolveSmem {
     unsigned char *stage0; // [MP_NW][stages][cbytes]
+    int off;               // byte offset of sy4 in dynamic shared memory
     float4 *sy4;           // [GMAX]   y, zero-padded
     float4 *sg4;           // [GMAX]   G as float (Cauchy pass), zero-padded
     double *sG, *sGp;      // [NMAX]   G_t, G_{t-1}
     double *sS, *sR;       // [NMAX]   s = y_t - y_{t-1}, r = G_t - G_{t-1} (the step's inputs)
-    double *sRed;          // [8]      the step's sums and maxima
-    FF *sGff;              // [NMAX + 1] the reduced sums as float pairs: -G, then F (converted in the step)
+    FF *sF;                // [MP_NW]  the warps' shares of F (of the curvature) as float pairs
     float *sYp;            // [NMAX]   y_{t-1}
     float *wred;           // [MP_NW][NMAX]
     float *sT, *sO, *sU;   // [256]
     uint64_t *bars;        // [MP_NW][PQ]
     uint32_t *ring_meta;   // [MP_NW][PQ][2] packed tiles: ring offset, bytes held
     int32_t *wlist;        // [MP_NW][WL_CAP][3] the warp's first tiles: tile, packed unit offset, units
+    // then FF [mp_cta_cap(NMAX)]: a column's slots staged for their sum (TailSmem::stage)
 };
 
-// Resident CTAs per SM the persistent solvers are compiled for (a register budget): more
-// CTAs for fewer apertures, whose tiles are small and whose warps wait on copies.
-__host__ __device__ constexpr int mp_min_ctas(int nmax) { return nmax <= 8 ? 4 : (nmax <= 24 ? 3 : (nmax <= 48 ? 2 : 1)); }
+// Resident CTAs per SM the persistent solvers are compiled for (a register budget): what
+// their shared memory (solve_smem) lets an SM hold, four up to 4 apertures, two up to 44
+// (the 48 of the last kernel of that class), else one.
+__host__ __device__ constexpr int mp_min_ctas(int nmax) { return nmax <= 4 ? 4 : (nmax <= 48 ? 2 : 1); }
+
+// CTAs a solve of nmax apertures has at most (room for a column's staged slots; up to 160 SMs).
+__host__ __device__ constexpr int mp_cta_cap(int nmax) { return 160 * mp_min_ctas(nmax); }
 
 // Copies in flight per warp at most (mbarriers per warp): the tile stages of whole tiles, or
 // the packed tiles that fit in the warp's byte ring.
@@ -448,12 +517,6 @@ constexpr int PQ = 8;
 // solve, so that issuing a copy and placing a tile's voxels wait on no global load); a
 // warp's tiles past the first WL_CAP are looked up in global memory.
 constexpr int WL_CAP = 64;
-
-template <int NMAX> __host__ __device__ constexpr size_t solve_fixed_smem() {
-    return 128 /* alignment slack */ + 2 * (NMAX / 4) * 16 + 4 * (size_t)NMAX * 8 + 8 * 8 + 8 * (size_t)(NMAX + 1) +
-           (size_t)NMAX * 4 +
-           (size_t)MP_NW * NMAX * 4 + 3 * 256 * 4 + (size_t)MP_NW * PQ * (8 + 8) + (size_t)MP_NW * WL_CAP * 12;
-}
 
 // Bulk copy of the warp's pipeline slot `it` (global tile-use index across passes).
 struct WarpPipe {
@@ -551,10 +614,10 @@ template <int NMAX, int MODE, bool PACKED>
 __device__ __forceinline__ bool solve_pass(const MPArgs &a, const SolveSmem &S, WarpPipe &P, int64_t &it,
                                            float *gacc, float &fs, float &fc) {
     constexpr int GMAX = NMAX / 4;
-    // From 56 to 72 apertures (one CTA per SM, registers to spare) a tile's groups stay in
+    // From 49 to 64 apertures (one CTA per SM, registers to spare) a tile's groups stay in
     // registers between the dose and the G shares, so its slot is refilled before the
     // objective; the Cauchy pass reads the slot once and refills at the same point.
-    constexpr bool KEEP = NMAX >= 56 && NMAX <= 72 && MODE == PASS_ITER;
+    constexpr bool KEEP = NMAX >= 56 && NMAX <= 64 && MODE == PASS_ITER;
     constexpr bool EARLY = KEEP || MODE == PASS_CAUCHY;
     const int G = (a.n + 3) >> 2;
     const int lane = threadIdx.x & 31;
@@ -670,40 +733,120 @@ __device__ __forceinline__ void warp_share_sums(const float *gacc, int n, float 
     }
 }
 
-// CTA sum of one float pair per thread (result in thread 0): warp butterflies, warps in order.
-__device__ FF block_ff(FF v, FF *sh) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) v = ff_add(v, ff_shfl_xor(v, d));
-    if (lane == 0) sh[wid] = v;
-    __syncthreads();
+// The warps' pairs sh[0 .. MP_NW) in order.
+__device__ __forceinline__ FF sum_warps_ff(const FF *sh) {
     FF t = sh[0];
-    if (threadIdx.x == 0)
-        for (int w = 1; w < MP_NW; ++w) t = ff_add(t, sh[w]);
-    __syncthreads();
+#pragma unroll
+    for (int w = 1; w < MP_NW; ++w) t = ff_add(t, sh[w]);
     return t;
 }
 
+// Exchange `tag` over n_col columns: every thread calls it after the CTA's slot of every column
+// has been written (by some of its threads).  A thread that wants column `want`'s sum gets it in
+// *out (want < 0: none).  epoch_src (elastic solver, else null): the owner of the last
+// column reads that word once, and a thread with want == n_col gets the value, the same in
+// every CTA, as the bits of out->hi.  Returns false in a thread whose wait ran out.
+__device__ __forceinline__ bool exchange_columns(const PState &ps, FF *stage, int n_col, unsigned tag, int want,
+                                                 FF *out, const unsigned *epoch_src) {
+    const int tid = threadIdx.x, lane = tid & 31, wid = warp_index();
+    const int cta = warp_uniform((int)ps.cta), n_cta = warp_uniform((int)ps.n_cta);
+    bool ok = true;
+    auto publish = [&](int k, FF v) { // a copy per lane
+        ulonglong2 *copy = ps.res + (size_t)lane * ps.rstride;
+        tagged_store(copy + k, v, tag);
+        if (epoch_src && k == n_col - 1) {
+            const unsigned e = __shfl_sync(0xffffffffu, lane == 0 ? *(const volatile unsigned *)epoch_src : 0u, 0);
+            tagged_store(copy + n_col, FF{__uint_as_float(e), 0.f}, tag);
+        }
+    };
+    if (n_cta >= n_col) { // a column or none per CTA: the CTA polls its slots
+        if (cta < n_col) {
+            FF v;
+            ok = column_sum_cta(ps.slots + (size_t)cta * ps.pstride, n_cta, tag, stage, wid, &v);
+            if (ok && wid == MP_NW - 1) publish(cta, v);
+        }
+    } else { // few CTAs: a warp per column, from the last warp down (the first ones poll results)
+        for (int k = cta + (MP_NW - 1 - wid) * n_cta; k < n_col; k += MP_NW * n_cta) {
+            FF v;
+            const bool got = column_sum(ps.slots + (size_t)k * ps.pstride, n_cta, tag, &v); // the same in every lane
+            ok = ok && got;
+            if (got) publish(k, v);
+        }
+    }
+    const ulonglong2 *res = ps.res + (size_t)(cta % RES_COPIES) * ps.rstride;
+    // polled a warp at a time, so that the warp stays together
+    if (__any_sync(0xffffffffu, want >= 0)) {
+        ulonglong2 w = make_ulonglong2(0, 0);
+        const long long t0 = clock64();
+        while (true) {
+            if (want >= 0) w = tagged_load(res + want);
+            if (__all_sync(0xffffffffu, want < 0 || tagged_ok(w, tag))) break;
+            if (__any_sync(0xffffffffu, clock64() - t0 > WAIT_LIMIT_CYCLES)) {
+                ok = false;
+                break;
+            }
+        }
+        if (want >= 0) *out = tagged_value(w);
+    }
+    return ok;
+}
+
+// The arrays of the solver's shared memory that the end of an iteration uses
+// (solve_layout's places, found from the solve's rounded aperture count).
+struct TailSmem {
+    float *y, *sg, *sYp, *wred;
+    double *sG, *sGp, *sS, *sR;
+    FF *sF, *stage;
+};
+__device__ __forceinline__ TailSmem tail_smem(const PState &ps) {
+    extern __shared__ __align__(128) unsigned char sm_raw[];
+    unsigned char *b = sm_raw + ps.off;
+    const int m = ps.nmax;
+    TailSmem S;
+    S.y = reinterpret_cast<float *>(b);
+    S.sg = S.y + m;
+    S.sG = reinterpret_cast<double *>(S.sg + m);
+    S.sGp = S.sG + m;
+    S.sS = S.sGp + m;
+    S.sR = S.sS + m;
+    S.sF = reinterpret_cast<FF *>(S.sR + m);
+    S.sYp = reinterpret_cast<float *>(S.sF + MP_NW);
+    S.wred = S.sYp + m;
+    S.stage = reinterpret_cast<FF *>(reinterpret_cast<unsigned char *>(S.wred + MP_NW * m + 3 * 256) +
+                                     MP_NW * PQ * (8 + 8) + MP_NW * WL_CAP * 12);
+    return S;
+}
+
+// The threads that take F and the elastic solver's epoch: in a warp without columns, so that
+// no warp runs the work of a column and of F one after the other.
+constexpr int F_THREAD = MP_NMAX, EPOCH_THREAD = MP_NMAX + 1;
+static_assert(F_THREAD % 32 == 0 && EPOCH_THREAD < MP_THREADS, "a warp of their own");
+
+enum { STEP_NEXT = 0, STEP_DONE = 1, STEP_CAUCHY = 2 };
+
 // Eq. 9-10 freeze, stopping tests, BB step length (FP64) and projected update, on the
-// shared-memory copy of the state, run by the whole CTA.  FP64 issues at a small
-// fraction of the FP32 rate on this GPU and one warp's chain of FP64 operations was
-// the step's cost, so the work is spread: one aperture per thread (freeze, s, r),
-// then one warp per sum or maximum (each lane over apertures l, l + 32, ... in
-// order, then a fixed butterfly), then thread 0 decides.  Every CTA runs it on
-// identical inputs.  Ends synchronised.
-template <int NMAX>
-__device__ void solve_step_cta(const MPArgs &a, const SolveSmem &S, PState &ps) {
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const int n = a.n, t = ps.t;
-    float *y = reinterpret_cast<float *>(S.sy4);
-    // FP64 issues at a small fraction of the FP32 rate on this GPU: the reduced float pairs
-    // are converted here, one column per thread, not one column per warp instruction
-    if (tid == MP_THREADS - 1) ps.F = ff_to_double(S.sGff[n]) + a.F_offset + (a.F_off_dev ? __ldcg(a.F_off_dev) : 0.0);
-    for (int k = tid; k < n; k += MP_THREADS) {
-        float yk = y[k];
-        const float l = lo_of(a, k), h = hi_of(a, k);
-        const FF gf = S.sGff[k]; // g = -(hi + lo): its sign from a float compare (the pair's sum is not rounded to 0)
-        double g = -ff_to_double(gf);
+// shared-memory copy of the state, run by the whole CTA; every CTA runs it on identical
+// inputs.  Thread k < n comes with column k's reduced pair (-G_k) in gf and its bounds,
+// thread F_THREAD with F; `ok` false in a thread whose exchange failed: then -1 everywhere.
+// Returns the same STEP_* in every thread; after STEP_NEXT y holds the next iterate.
+//
+// What bounds it: a chain of FP64 operations, which issue at a small fraction of the
+// FP32 rate on this GPU.  So the work is spread (one aperture per thread, one warp per
+// sum, the tests and the step size each in a warp of its own) with one CTA barrier per
+// stage, every thread decides for itself from the stage's results, and no stage loads
+// from global memory (the tile constant, which each step used to read, cost it an L2
+// access on this chain).
+__device__ __forceinline__ int solve_step_cta(PState &ps, const TailSmem &S, FF gf, float l, float h, bool ok) {
+    const int tid = threadIdx.x, lane = tid & 31, wid = warp_index();
+    const int n = warp_uniform(ps.n), t = ps.t;
+    float *y = S.y;
+    float yk = 0.f;
+    double g = 0.0;
+    if (tid == F_THREAD) ps.F = ff_to_double(gf) + ps.F_offset + ps.F_off;
+    if (tid < n) {
+        yk = y[tid];
+        // g = -(hi + lo): its sign from a float compare (the pair's sum is not rounded to 0)
+        g = -ff_to_double(gf);
         if (yk <= l && gf.hi < -gf.lo) {
             yk = l;
             g = 0.0;
@@ -711,30 +854,45 @@ __device__ void solve_step_cta(const MPArgs &a, const SolveSmem &S, PState &ps) 
             yk = h;
             g = 0.0;
         }
-        y[k] = yk;
-        S.sG[k] = g;
+        y[tid] = yk;
+        S.sG[tid] = g;
         if (t > 0) {
-            S.sS[k] = (double)yk - (double)S.sYp[k];
-            S.sR[k] = g - S.sGp[k];
+            S.sS[tid] = (double)yk - (double)S.sYp[tid];
+            S.sR[tid] = g - S.sGp[tid];
         }
     }
-    __syncthreads();
+    if (__syncthreads_or(!ok)) return -1;
     // Warp 0: the four sums, eight lanes each (lanes 8q .. 8q + 7: 0 G.G, 1 s.s, 2 s.r,
     // 3 r.r), lane j of a group over apertures j, j + 8, ... in order, then a fixed
     // butterfly of the group: one warp's FP64 instructions serve all four.  Warp 1: the
     // maxima |s| (lanes 0-15) and |y| (lanes 16-31) as integer maxima of the bit
-    // patterns of non-negative values (the order of their values), off the FP64 pipe.
-    // (the group's operands come through selected pointers, so that the warp does not
-    // diverge; at t = 0 the groups other than G.G read stale values, never used)
+    // patterns of non-negative values (the order of their values), off the FP64 pipe,
+    // and with them the step test.  Warp 2: the relative-change test, which needs F only.
+    // (the groups' operands are offsets into one array and the trip count is the warp's, so
+    // that the warp does not run the groups one after the other; at t = 0 the groups other
+    // than G.G read stale values, never used)
     if (wid == 0) {
         const int q = lane >> 3, j = lane & 7;
-        const double *xa = q == 0 ? S.sG : (q == 3 ? S.sR : S.sS);
-        const double *za = q == 2 ? S.sR : xa;
+        const int m = ps.nmax, ox = (q == 0 ? 0 : (q == 3 ? 3 : 2)) * m + j, oz = (q == 0 ? 0 : (q == 1 ? 2 : 3)) * m + j;
         double v = 0.0;
-        for (int k = j; k < n; k += 8) v += xa[k] * za[k];
+        for (int k = 0; k < n; k += 8) { // entries past n (up to 7, sR's in sF) are read and left out
+            const double p = fma(S.sG[ox + k], S.sG[oz + k], v);
+            v = k + j < n ? p : v;
+        }
 #pragma unroll
         for (int d = 4; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
-        if (j == 0) S.sRed[q] = v;
+        const double ss = __shfl_sync(0xffffffffu, v, 8), sr = __shfl_sync(0xffffffffu, v, 16),
+                     rr = __shfl_sync(0xffffffffu, v, 24);
+        if (lane == 0) {
+            ps.gg = t == 0 ? v : ps.gg;
+            if (t > 0) {
+                double delta;
+                if (sr <= 0.0) delta = ps.opts.delta_max * ps.delta0;
+                else if (t & 1) delta = sr / rr;
+                else delta = ss / sr;
+                ps.delta = fmin(fmax(delta, ps.opts.delta_min * ps.delta0), ps.opts.delta_max * ps.delta0);
+            }
+        }
     } else if (wid == 1) {
         const bool ys = lane >= 16;
         const int j = lane & 15;
@@ -747,84 +905,133 @@ __device__ void solve_step_cta(const MPArgs &a, const SolveSmem &S, PState &ps) 
         }
 #pragma unroll
         for (int d = 8; d > 0; d >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, d));
-        if (j == 0) S.sRed[ys ? 5 : 4] = ys ? (double)__uint_as_float((unsigned)m) : __longlong_as_double((long long)m);
-    }
-    __syncthreads();
-    // the two stopping tests and the BB step size, each by lane 0 of its own warp (their
-    // FP64 chains run side by side); thread 0 then decides in the sequential order
-    if (lane == 0 && wid < 3) {
-        const double ss = S.sRed[1], sr = S.sRed[2], rr = S.sRed[3], dy = S.sRed[4], ymax = S.sRed[5];
-        if (wid == 0) {
-            const double F = ps.F;
-            ps.stop_rel = t >= 5 && fabs(ps.F_hist[(t - 5) % 6] - F) <= a.opts.rel_tol5 * F;
-        } else if (wid == 1) {
-            ps.stop_step = t >= 1 && dy <= a.opts.step_tol * fmax(1.0, ymax);
-        } else if (t > 0) {
-            double delta;
-            if (sr <= 0.0) delta = a.opts.delta_max * ps.delta0;
-            else if (t & 1) delta = sr / rr;
-            else delta = ss / sr;
-            ps.delta_c = fmin(fmax(delta, a.opts.delta_min * ps.delta0), a.opts.delta_max * ps.delta0);
+        const unsigned long long my = __shfl_sync(0xffffffffu, m, 16);
+        if (lane == 0) {
+            const double dy = __longlong_as_double((long long)m), ymax = (double)__uint_as_float((unsigned)my);
+            ps.stop_step = t >= 1 && dy <= ps.opts.step_tol * fmax(1.0, ymax);
         }
+    } else if (wid == 2 && lane == 0) {
+        const double F = ps.F;
+        ps.stop_rel = t >= 5 && fabs(ps.F_hist[(t - 5) % 6] - F) <= ps.opts.rel_tol5 * F;
+        ps.F_hist[t % 6] = F; // (t - 5) % 6 is another entry
     }
     __syncthreads();
-    if (tid == 0) {
-        const double gg = S.sRed[0];
-        ps.decided = 1;
-        ps.F_hist[t % 6] = ps.F;
-        if (ps.stop_rel) {
+    int stop = 0;
+    if (ps.stop_rel) stop = VMAT_STOP_REL;
+    else if (ps.stop_step) stop = VMAT_STOP_STEP;
+    else if (t == ps.opts.max_iter - 1) stop = VMAT_STOP_MAXIT;
+    else if (t == 0 && ps.gg == 0.0) stop = VMAT_STOP_GRAD0;
+    if (stop) {
+        if (tid == 0) {
             ps.done = 1;
-            ps.stop = VMAT_STOP_REL;
-        } else if (ps.stop_step) {
-            ps.done = 1;
-            ps.stop = VMAT_STOP_STEP;
-        } else if (t == a.opts.max_iter - 1) {
-            ps.done = 1;
-            ps.stop = VMAT_STOP_MAXIT;
-        } else if (t == 0) {
-            if (gg == 0.0) {
-                ps.done = 1;
-                ps.stop = VMAT_STOP_GRAD0;
-            } else {
-                ps.gg = gg;
-                ps.decided = 2; // the first step is the Cauchy step (needs DA G)
-            }
-        } else {
-            ps.delta = ps.delta_c;
-            ps.decided = 0;
+            ps.stop = stop;
         }
+        __syncthreads();
+        return STEP_DONE;
+    }
+    if (t == 0) return STEP_CAUCHY; // the first step's length needs DA G
+    if (tid < n) {
+        S.sYp[tid] = yk;
+        S.sGp[tid] = g;
+        const double yn = (double)yk - ps.delta * g;
+        y[tid] = fminf(fmaxf((float)yn, l), h);
     }
     __syncthreads();
+    return STEP_NEXT;
 }
 
-// y <- clamp(y - delta G) after saving (y, G) as the previous iterate, one aperture
-// per thread (the whole CTA).  Ends synchronised.
-__device__ void solve_take_step_cta(const MPArgs &a, const SolveSmem &S, double delta) {
-    float *y = reinterpret_cast<float *>(S.sy4);
-    for (int k = threadIdx.x; k < a.n; k += MP_THREADS) {
-        const float yk = y[k];
-        S.sYp[k] = yk;
-        S.sGp[k] = S.sG[k];
-        const double yn = (double)yk - delta * S.sG[k];
-        y[k] = fminf(fmaxf((float)yn, lo_of(a, k)), hi_of(a, k));
+// The end of an iteration, after every warp has written its G shares to wred: this CTA's
+// partials of every column and of F (fs - fc per lane), their sums over the CTAs, the step.
+// Returns STEP_* (the same in every CTA), -1 when a wait ran out.  Not inlined: the pass
+// keeps its registers (inlined, the two together spilled inside the pass).
+__device__ __noinline__ int solve_tail(float fs, float fc) {
+    PState &ps = solve_state();
+    const TailSmem S = tail_smem(ps);
+    const int tid = threadIdx.x, lane = tid & 31, wid = warp_index();
+    const int n = warp_uniform(ps.n), m = ps.nmax;
+    const float l = tid < n && ps.lo ? ps.lo[tid] : 0.f, h = tid < n && ps.hi ? ps.hi[tid] : INFINITY;
+    const FF fw = warp_ff(FF{fs, -fc});
+    if (lane == 0) S.sF[wid] = fw;
+    const unsigned tag = ps.tag + 1;
+    __syncthreads();
+    if (ps.abort) return -1;
+    FF v{0.f, 0.f};
+    if (tid < n) {
+        v = FF{S.wred[tid], 0.f};
+#pragma unroll
+        for (int w = 1; w < MP_NW; ++w) v = ff_add(v, FF{S.wred[w * m + tid], 0.f});
+    } else if (tid == F_THREAD) {
+        v = sum_warps_ff(S.sF);
+    }
+    const int col = tid < n ? tid : (tid == F_THREAD ? n : -1);
+    if (col >= 0) tagged_store(ps.slots + (size_t)col * ps.pstride + ps.cta, v, tag);
+    const int want = ps.epoch_src && tid == EPOCH_THREAD ? n + 1 : col;
+    const bool ok = exchange_columns(ps, S.stage, n + 1, tag, want, &v, ps.epoch_src);
+    if (tid == EPOCH_THREAD) {
+        ps.epoch = __float_as_uint(v.hi);
+        ps.tag = tag; // read above, before the barrier; next read after the step's barriers
+        ++ps.passes;
+    }
+    return solve_step_cta(ps, S, v, l, h, ok);
+}
+
+// The end of the Cauchy pass (curvature terms cs - cc per lane): delta0 = G.G / (2 sum_i w_i
+// (DA G)_i^2) and the first step.  Returns STEP_NEXT, STEP_DONE (flat) or -1.
+__device__ __noinline__ int solve_cauchy_tail(float cs, float cc) {
+    PState &ps = solve_state();
+    const TailSmem S = tail_smem(ps);
+    const int tid = threadIdx.x, lane = tid & 31, wid = warp_index();
+    const int n = ps.n;
+    const float l = tid < n && ps.lo ? ps.lo[tid] : 0.f, h = tid < n && ps.hi ? ps.hi[tid] : INFINITY;
+    const FF cw = warp_ff(FF{cs, -cc});
+    if (lane == 0) S.sF[wid] = cw;
+    const unsigned tag = ps.tag + 1;
+    __syncthreads();
+    if (ps.abort) return -1;
+    FF c{0.f, 0.f};
+    if (tid == 0) tagged_store(ps.slots + ps.cta, sum_warps_ff(S.sF), tag);
+    const bool ok = exchange_columns(ps, S.stage, 1, tag, tid == 0 ? 0 : -1, &c, nullptr);
+    if (tid == 0 && ok) {
+        ps.tag = tag;
+        ++ps.passes;
+        const double curv = 2.0 * ff_to_double(c);
+        if (curv == 0.0) {
+            ps.done = 1;
+            ps.stop = VMAT_STOP_FLAT;
+        } else {
+            ps.delta0 = ps.gg / curv;
+        }
+    }
+    if (__syncthreads_or(!ok)) return -1;
+    if (ps.done) return STEP_DONE;
+    if (tid < n) {
+        const float yk = S.y[tid];
+        S.sYp[tid] = yk;
+        S.sGp[tid] = S.sG[tid];
+        const double yn = (double)yk - ps.delta0 * S.sG[tid];
+        S.y[tid] = fminf(fmaxf((float)yn, l), h);
     }
     __syncthreads();
+    return STEP_NEXT;
 }
 
 // Shared-memory layout of the solver for NMAX apertures and `stages` tiles per warp.
-template <int NMAX> __device__ __forceinline__ SolveSmem solve_layout(unsigned char *sm, int stages, uint32_t cbytes) {
+// sm_base: the start of dynamic shared memory, sm: its first 128-byte boundary.
+template <int NMAX>
+__device__ __forceinline__ SolveSmem solve_layout(const unsigned char *sm_base, unsigned char *sm, int stages,
+                                                  uint32_t cbytes) {
     constexpr int GMAX = NMAX / 4;
     SolveSmem S;
     S.stage0 = sm;
     S.sy4 = reinterpret_cast<float4 *>(sm + (size_t)MP_NW * stages * cbytes);
+    S.off = (int)(smem_u32(S.sy4) - smem_u32(sm_base));
     S.sg4 = S.sy4 + GMAX;
     S.sG = reinterpret_cast<double *>(S.sg4 + GMAX);
     S.sGp = S.sG + NMAX;
     S.sS = S.sGp + NMAX;
     S.sR = S.sS + NMAX;
-    S.sRed = S.sR + NMAX;
-    S.sGff = reinterpret_cast<FF *>(S.sRed + 8);
-    S.sYp = reinterpret_cast<float *>(S.sGff + NMAX + 1);
+    S.sF = reinterpret_cast<FF *>(S.sR + NMAX);
+    S.sYp = reinterpret_cast<float *>(S.sF + MP_NW);
     S.wred = S.sYp + NMAX;
     S.sT = S.wred + MP_NW * NMAX;
     S.sO = S.sT + 256;
@@ -836,13 +1043,17 @@ template <int NMAX> __device__ __forceinline__ SolveSmem solve_layout(unsigned c
 }
 
 // Loads one problem's tables and state into shared memory: a fresh start (y from
-// a.y, clamped by the init kernel) or, for the elastic solver, the state a
+// a.y, projected onto the box) or, for the elastic solver, the state a
 // previous epoch saved (t, F history, step scale, y, y_prev, G_prev).
-template <int NMAX> __device__ void solve_load(const MPArgs &a, const SolveSmem &S, PState &ps, bool resume) {
+template <int NMAX>
+__device__ void solve_load(const MPArgs &a, const SolveSmem &S, bool resume, unsigned cta, unsigned n_cta,
+                           const unsigned *epoch_src) {
     constexpr int GMAX = NMAX / 4;
+    PState &ps = solve_state();
     const int n = a.n, tid = threadIdx.x;
     for (int k = tid; k < 4 * GMAX; k += MP_THREADS) {
-        reinterpret_cast<float *>(S.sy4)[k] = k < n ? a.y[k] : 0.f;
+        // the start projected onto the box (a saved iterate lies in it)
+        reinterpret_cast<float *>(S.sy4)[k] = k < n ? fminf(fmaxf(a.y[k], lo_of(a, k)), hi_of(a, k)) : 0.f;
         reinterpret_cast<float *>(S.sg4)[k] = 0.f;
     }
     for (int k = tid; k < a.n_struct; k += MP_THREADS) {
@@ -858,6 +1069,22 @@ template <int NMAX> __device__ void solve_load(const MPArgs &a, const SolveSmem 
     if (tid == 0) {
         PState z = {};
         ps = z;
+        ps.tag = __ldcg(a.tag);
+        ps.F_off = a.F_off_dev ? __ldcg(a.F_off_dev) : 0.0;
+        ps.n = n;
+        ps.nmax = NMAX;
+        ps.off = S.off;
+        ps.cta = cta;
+        ps.n_cta = n_cta;
+        ps.slots = a.slots;
+        ps.res = a.res;
+        ps.pstride = a.pstride;
+        ps.rstride = a.rstride;
+        ps.epoch_src = epoch_src;
+        ps.lo = a.lo;
+        ps.hi = a.hi;
+        ps.opts = a.opts;
+        ps.F_offset = a.F_offset;
         if (resume) {
             for (int i = 0; i < 6; ++i) ps.F_hist[i] = a.st->F_hist[i];
             ps.F = a.st->F;
@@ -869,8 +1096,13 @@ template <int NMAX> __device__ void solve_load(const MPArgs &a, const SolveSmem 
     __syncthreads();
 }
 
+// A solve leaves *tag past every tag any of its CTAs has used (they are at most one
+// exchange apart), whether it ends, hands over or gives up.
+constexpr unsigned TAG_GAP = 4;
+
 // The state a later epoch resumes from (one CTA writes it).
-template <int NMAX> __device__ void solve_save(const MPArgs &a, const SolveSmem &S, const PState &ps) {
+template <int NMAX> __device__ void solve_save(const MPArgs &a, const SolveSmem &S) {
+    const PState &ps = solve_state();
     const float *y = reinterpret_cast<const float *>(S.sy4);
     for (int k = threadIdx.x; k < a.n; k += MP_THREADS) {
         a.y[k] = y[k];
@@ -884,12 +1116,14 @@ template <int NMAX> __device__ void solve_save(const MPArgs &a, const SolveSmem 
         a.st->gg = ps.gg;
         a.st->t = ps.t;
         a.st->started = 1;
+        *a.tag = ps.tag + TAG_GAP;
     }
     __threadfence();
 }
 
 // The end of a solve (one CTA): y, the report and the iteration count.
-template <int NMAX> __device__ void solve_finish(const MPArgs &a, const SolveSmem &S, const PState &ps, bool ok) {
+template <int NMAX> __device__ void solve_finish(const MPArgs &a, const SolveSmem &S, bool ok) {
+    const PState &ps = solve_state();
     const float *y = reinterpret_cast<const float *>(S.sy4);
     if (ok)
         for (int k = threadIdx.x; k < a.n; k += MP_THREADS) a.y[k] = y[k];
@@ -900,6 +1134,7 @@ template <int NMAX> __device__ void solve_finish(const MPArgs &a, const SolveSme
         a.st->stop = ok ? ps.stop : VMAT_STOP_MAXIT;
         a.st->iters = ps.t + 1;
         a.st->delta0 = ps.delta0;
+        *a.tag = ps.tag + TAG_GAP;
         if (ok && a.iters_acc) *a.iters_acc += ps.t + 1;
         if (ok && a.bytes_acc) { // each pass reads the tiles' labels and columns and writes (or reads) their dose
             const int64_t tiles = a.tiles ? min64((int64_t)max(__ldcg(a.n_live), 0), a.n_wtiles) : a.n_wtiles;
@@ -913,31 +1148,16 @@ template <int NMAX> __device__ void solve_finish(const MPArgs &a, const SolveSme
 
 enum { LOOP_DONE = 0, LOOP_ABORT = 1, LOOP_REBALANCE = 2 };
 
-// BB iterations of one problem as CTA `cta` of n_cta, until a stopping rule
-// (LOOP_DONE), a wait that ran out (LOOP_ABORT) or, for the elastic solver
-// (epoch_src non-null), a change of the batch epoch seen at the second barrier of
-// an iteration (LOOP_REBALANCE, after this CTA has saved the state if cta == 0).
+// BB iterations of one problem, until a stopping rule
+// (LOOP_DONE), a wait that ran out (LOOP_ABORT) or, for the elastic solver, a change of the batch epoch seen at an iteration's exchange
+// (LOOP_REBALANCE, after this CTA has saved the state if cta == 0).
 template <int NMAX>
-__device__ int solve_loop(const MPArgs &a, const SolveSmem &S, WarpPipe &P, PState &ps, int64_t &it,
-                          const unsigned cta, const unsigned n_cta, const unsigned *epoch_src, unsigned epoch_local) {
+__device__ __forceinline__ int solve_loop(const MPArgs &a, const SolveSmem &S, WarpPipe &P, int64_t &it, bool elastic,
+                                          unsigned epoch_local) {
     constexpr int GMAX = NMAX / 4;
-    __shared__ FF shff[MP_NW];
-    __shared__ int abort_s;
-    const int n = a.n;
+    PState &ps = solve_state();
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    if (tid == 0) abort_s = 0;
-    __syncthreads();
-    // the single-problem solve (no epochs) keeps its CTAs: its barriers count arrivals
-    // on one growing counter; the elastic solver's use the counter and generation pair
-    unsigned bar_e = 0;
-    auto sync_grid = [&](bool snap) -> bool {
-        if (!epoch_src) return grid_sync_count(a.bar_count, ++bar_e * n_cta);
-        return snap ? grid_sync(a.bar_count, a.bar_gen, n_cta, a.epoch_snap, epoch_src)
-                    : grid_sync(a.bar_count, a.bar_gen, n_cta);
-    };
     float gacc[NMAX];
-    FF *part = reinterpret_cast<FF *>(a.part);
-    FF *cpart = reinterpret_cast<FF *>(a.cpart);
     while (true) {
         // ---- pass: z = DA y, g, F and this CTA's shares of G = -DA^T g
 #pragma unroll
@@ -945,109 +1165,25 @@ __device__ int solve_loop(const MPArgs &a, const SolveSmem &S, WarpPipe &P, PSta
         float fs = 0.f, fc = 0.f;
         const bool pass_ok = P.n_my == 0 || (P.poff ? solve_pass<NMAX, PASS_ITER, true>(a, S, P, it, gacc, fs, fc)
                                                     : solve_pass<NMAX, PASS_ITER, false>(a, S, P, it, gacc, fs, fc));
-        if (tid == 0) ++ps.passes;
-        if (!pass_ok && lane == 0) atomicOr(&abort_s, 1);
-        warp_share_sums<NMAX>(gacc, n, S.wred + wid * NMAX, lane);
-        const FF fb = block_ff(FF{fs, -fc}, shff); // includes a __syncthreads after wred
-        // this CTA's partials, column-major by CTA, in the buffer of this iteration's parity: a CTA
-        // writes buffer b again two iterations later, after the barrier that every CTA reaches only
-        // once it has read buffer b
-        FF *pb = part + (size_t)(ps.t & 1) * (n + 1) * a.pstride;
-        for (int k = tid; k < n; k += MP_THREADS) {
-            FF sum{S.wred[k], 0.f};
-            for (int w = 1; w < MP_NW; ++w) sum = ff_add(sum, FF{S.wred[w * NMAX + k], 0.f});
-            pb[(size_t)k * a.pstride + cta] = sum;
-        }
-        if (tid == 0) pb[(size_t)n * a.pstride + cta] = fb;
-        if (abort_s || !sync_grid(true)) return LOOP_ABORT;
-        // ---- every CTA reduces every column itself: warp w takes columns w, w + MP_NW, ...,
-        // CB at a time with eight loads per column in flight per lane (every load of the group
-        // issued before the first add; CB grows with NMAX, whose kernels have fewer CTAs per SM
-        // and more columns per warp, and stays 1 where registers set the CTAs per SM); lane l
-        // sums CTAs l, l + 32, ... in order, then a fixed butterfly: the same G and F in every
-        // CTA, with no second barrier
-        constexpr int CB = NMAX >= 56 ? 4 : (NMAX >= 32 ? 2 : 1);
-        for (int k0 = wid; k0 <= n; k0 += MP_NW * CB) {
-            FF v[CB];
-#pragma unroll
-            for (int j = 0; j < CB; ++j) v[j] = FF{0.f, 0.f};
-            for (unsigned b0 = lane; b0 < n_cta; b0 += 32 * 8) {
-                float2 q[CB][8];
-#pragma unroll
-                for (int j = 0; j < CB; ++j) {
-                    const int k = k0 + MP_NW * j;
-                    const float2 *col = reinterpret_cast<const float2 *>(pb + (size_t)min(k, n) * a.pstride);
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) {
-                        const unsigned b = b0 + 32u * u;
-                        q[j][u] = k <= n && b < n_cta ? __ldcg(col + b) : make_float2(0.f, 0.f);
-                    }
-                }
-#pragma unroll
-                for (int j = 0; j < CB; ++j)
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) v[j] = ff_add(v[j], FF{q[j][u].x, q[j][u].y});
-            }
-#pragma unroll
-            for (int d = 16; d > 0; d >>= 1)
-#pragma unroll
-                for (int j = 0; j < CB; ++j) v[j] = ff_add(v[j], ff_shfl_xor(v[j], d));
-            if (lane == 0) { // float pairs: the step converts them a column per thread
-#pragma unroll
-                for (int j = 0; j < CB; ++j) {
-                    const int k = k0 + MP_NW * j;
-                    if (k <= n) S.sGff[k] = v[j];
-                }
-            }
-        }
-        __syncthreads();
-        solve_step_cta<NMAX>(a, S, ps);
-        if (ps.decided == 0) solve_take_step_cta(a, S, ps.delta);
-        if (ps.decided == 2) {
-            // ---- Cauchy step: delta0 = G.G / (2 sum_i w_i (DA G)_i^2)
+        if (!pass_ok && lane == 0) ps.abort = 1;
+        warp_share_sums<NMAX>(gacc, a.n, S.wred + wid * NMAX, lane);
+        int step = solve_tail(fs, fc);
+        if (step == STEP_CAUCHY) { // the first step's length needs DA G
             for (int k = tid; k < 4 * GMAX; k += MP_THREADS)
-                reinterpret_cast<float *>(S.sg4)[k] = k < n ? (float)S.sG[k] : 0.f;
+                reinterpret_cast<float *>(S.sg4)[k] = k < a.n ? (float)S.sG[k] : 0.f;
             __syncthreads();
-            float cs = 0.f, cc = 0.f;
-            const bool c_ok = P.n_my == 0 || (P.poff ? solve_pass<NMAX, PASS_CAUCHY, true>(a, S, P, it, gacc, cs, cc)
-                                                      : solve_pass<NMAX, PASS_CAUCHY, false>(a, S, P, it, gacc, cs, cc));
-            if (tid == 0) ++ps.passes;
-            if (!c_ok && lane == 0) atomicOr(&abort_s, 1);
-            const FF cb = block_ff(FF{cs, -cc}, shff);
-            if (tid == 0) cpart[cta] = cb;
-            if (abort_s || !sync_grid(false)) return LOOP_ABORT;
-            if (wid == 0) {
-                FF v{0.f, 0.f};
-                for (unsigned b0 = lane; b0 < n_cta; b0 += 32 * 8) {
-                    float2 q[8];
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) {
-                        const unsigned b = b0 + 32u * u;
-                        q[u] = b < n_cta ? __ldcg(reinterpret_cast<const float2 *>(cpart) + b) : make_float2(0.f, 0.f);
-                    }
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) v = ff_add(v, FF{q[u].x, q[u].y});
-                }
-#pragma unroll
-                for (int d = 16; d > 0; d >>= 1) v = ff_add(v, ff_shfl_xor(v, d));
-                const double curv = 2.0 * ff_to_double(v);
-                if (lane == 0) {
-                    if (curv == 0.0) {
-                        ps.done = 1;
-                        ps.stop = VMAT_STOP_FLAT;
-                    } else {
-                        ps.delta0 = ps.gg / curv;
-                    }
-                }
-            }
-            __syncthreads();
-            if (!ps.done) solve_take_step_cta(a, S, ps.delta0);
+            fs = fc = 0.f;
+            const bool c_ok = P.n_my == 0 || (P.poff ? solve_pass<NMAX, PASS_CAUCHY, true>(a, S, P, it, gacc, fs, fc)
+                                                      : solve_pass<NMAX, PASS_CAUCHY, false>(a, S, P, it, gacc, fs, fc));
+            if (!c_ok && lane == 0) ps.abort = 1;
+            step = solve_cauchy_tail(fs, fc);
         }
-        if (ps.done) return LOOP_DONE;
-        if (tid == 0) ++ps.t;
-        __syncthreads();
-        if (epoch_src && __ldcg(a.epoch_snap) != epoch_local) { // the same word for every CTA of the problem
-            if (cta == 0) solve_save<NMAX>(a, S, ps);
+        if (step < 0) return LOOP_ABORT;
+        if (step == STEP_DONE) return LOOP_DONE;
+        if (tid == 0) ++ps.t; // next read after the tail's first barrier
+        if (elastic && ps.epoch != epoch_local) { // the same word for every CTA of the problem
+            __syncthreads();
+            if (ps.cta == 0) solve_save<NMAX>(a, S);
             return LOOP_REBALANCE;
         }
     }
@@ -1122,23 +1258,23 @@ __device__ __forceinline__ void pipe_init(WarpPipe &P, const SolveSmem &S, int s
 }
 
 template <int NMAX>
-__global__ void __launch_bounds__(MP_THREADS, mp_min_ctas(NMAX)) mp_solve_kernel(MPArgs a, int stages, int keep_in_l2) {
+__global__ void __launch_bounds__(MP_THREADS, mp_min_ctas(NMAX))
+    mp_solve_kernel(const __grid_constant__ MPArgs a, int stages, int keep_in_l2) {
     if (a.skip && *a.skip) return; // the same flag for every CTA: all return together
     extern __shared__ __align__(128) unsigned char sm_raw[];
-    __shared__ PState ps;
     // align the staging area explicitly: static shared memory may shift the dynamic region
     unsigned char *sm = sm_raw + ((128u - (smem_u32(sm_raw) & 127u)) & 127u);
     const uint32_t cbytes = (uint32_t)wt_copy_bytes(a.n);
-    const SolveSmem S = solve_layout<NMAX>(sm, stages, cbytes);
+    const SolveSmem S = solve_layout<NMAX>(sm_raw, sm, stages, cbytes);
     WarpPipe P;
     pipe_init(P, S, stages, cbytes, keep_in_l2);
-    solve_load<NMAX>(a, S, ps, false); // ends with a __syncthreads (barriers initialised)
+    solve_load<NMAX>(a, S, false, blockIdx.x, gridDim.x, nullptr); // ends with a __syncthreads (barriers initialised)
     int64_t it = 0;
     pipe_start(P, a, blockIdx.x, gridDim.x, it);
-    const int r = solve_loop<NMAX>(a, S, P, ps, it, blockIdx.x, gridDim.x, nullptr, 0u);
+    const int r = solve_loop<NMAX>(a, S, P, it, false, 0u);
     if (r == LOOP_ABORT && threadIdx.x == 0) atomicOr(a.status, DEV_TIMEOUT);
     pipe_drain(P, it);
-    if (blockIdx.x == 0) solve_finish<NMAX>(a, S, ps, r != LOOP_ABORT);
+    if (blockIdx.x == 0) solve_finish<NMAX>(a, S, r != LOOP_ABORT);
 }
 
 __device__ bool batch_sync(unsigned *gctl, unsigned n_cta, const MPArgs *args, int n_plans) {
@@ -1192,12 +1328,11 @@ __global__ void __launch_bounds__(MP_THREADS, mp_min_ctas(NMAX))
                             int32_t n, unsigned *gctl, int stages, int keep_in_l2) {
     extern __shared__ __align__(128) unsigned char sm_raw[];
     __shared__ MPArgs sa;
-    __shared__ PState ps;
     __shared__ int sp, sc, sn, resume_s;
     __shared__ unsigned epoch_s;
     unsigned char *sm = sm_raw + ((128u - (smem_u32(sm_raw) & 127u)) & 127u);
     const uint32_t cbytes = (uint32_t)wt_copy_bytes(n);
-    const SolveSmem S = solve_layout<NMAX>(sm, stages, cbytes);
+    const SolveSmem S = solve_layout<NMAX>(sm_raw, sm, stages, cbytes);
     WarpPipe P;
     pipe_init(P, S, stages, cbytes, keep_in_l2);
     __syncthreads();
@@ -1248,19 +1383,19 @@ __global__ void __launch_bounds__(MP_THREADS, mp_min_ctas(NMAX))
         }
         __syncthreads();
         const unsigned c = (unsigned)sc, nc = (unsigned)sn;
-        solve_load<NMAX>(sa, S, ps, resume_s != 0);
+        solve_load<NMAX>(sa, S, resume_s != 0, c, nc, gctl + 2);
         pipe_start(P, sa, c, nc, it);
-        const int r = solve_loop<NMAX>(sa, S, P, ps, it, c, nc, gctl + 2, epoch_local);
+        const int r = solve_loop<NMAX>(sa, S, P, it, true, epoch_local);
         pipe_drain(P, it);
         if (P.n_my > 0) it += stages; // the drained slots were issued (a warp without tiles issued none)
         if (r == LOOP_ABORT) {
             ok = false;
             if (threadIdx.x == 0) atomicOr(sa.status, DEV_TIMEOUT);
-            if (c == 0) solve_finish<NMAX>(sa, S, ps, false);
+            if (c == 0) solve_finish<NMAX>(sa, S, false);
             break;
         }
         if (r == LOOP_DONE && c == 0) {
-            solve_finish<NMAX>(sa, S, ps, true);
+            solve_finish<NMAX>(sa, S, true);
             if (threadIdx.x == 0) atomicAdd(gctl + 2, 1u);
         }
         if (!batch_sync(gctl, gridDim.x, args, n_plans)) {
@@ -1292,9 +1427,6 @@ __global__ void mp_init_batched_kernel(const MPArgs *__restrict__ args, int32_t 
     if (threadIdx.x == 0) {
         BBState st = {};
         *a.st = st;
-        *a.bar_count = 0u;
-        *a.bar_gen = 0u;
-        *a.epoch_snap = 0u;
     }
 }
 
@@ -1709,19 +1841,20 @@ vmat_status mp_write_labels(const uint8_t *sid, int32_t V, int64_t wstride, floa
     return VMAT_OK;
 }
 
-static int solve_nmax(int n) { return ((n + 7) / 8) * 8; }
+static int solve_nmax(int n) { return n <= 4 ? 4 : ((n + 7) / 8) * 8; }
 static size_t solve_fixed(int n) {
     const int nmax = solve_nmax(n);
-    return 128 /* alignment slack */ + 2 * (size_t)(nmax / 4) * 16 + 4 * (size_t)nmax * 8 + 8 * 8 +
-           8 * (size_t)(nmax + 1) + (size_t)nmax * 4 + (size_t)MP_NW * nmax * 4 + 3 * 256 * 4 + (size_t)MP_NW * PQ * (8 + 8) +
-           (size_t)MP_NW * WL_CAP * 12;
+    return 128 /* alignment slack */ + 2 * (size_t)(nmax / 4) * 16 + 4 * (size_t)nmax * 8 + MP_NW * sizeof(FF) +
+           (size_t)nmax * 4 + (size_t)MP_NW * nmax * 4 + 3 * 256 * 4 + (size_t)MP_NW * PQ * (8 + 8) +
+           (size_t)MP_NW * WL_CAP * 12 + (size_t)mp_cta_cap(nmax) * sizeof(FF);
 }
 static size_t solve_smem(int n, int stages) { return solve_fixed(n) + (size_t)stages * MP_NW * wt_copy_bytes(n); }
 // Tiles in flight per warp: as many as fit (up to 8) in ~110 KB, so that two CTAs
-// share an SM; where not even two fit there, up to the per-CTA limit (one CTA per SM).
+// share an SM (in 53 KB up to 4 apertures: four CTAs); where not even two fit there, up to
+// the per-CTA limit (one CTA per SM).
 static int solve_stages(int n) {
     const size_t per = MP_NW * wt_copy_bytes(n);
-    const size_t small = 110 * 1024;
+    const size_t small = (n <= 4 ? 53 : 110) * 1024;
     const size_t st = solve_fixed(n) + 2 * per <= small ? (small - solve_fixed(n)) / per
                                                         : (MP_SMEM_LIMIT - solve_fixed(n)) / per;
     return (int)std::min<size_t>(8, st);
@@ -1730,7 +1863,7 @@ static int solve_stages(int n) {
 using SolveFn = void (*)(MPArgs, int, int);
 static SolveFn solve_kernel_for(int n) {
     switch ((n + 7) / 8) {
-    case 1: return mp_solve_kernel<8>;
+    case 1: return n <= 4 ? mp_solve_kernel<4> : mp_solve_kernel<8>;
     case 2: return mp_solve_kernel<16>;
     case 3: return mp_solve_kernel<24>;
     case 4: return mp_solve_kernel<32>;
@@ -1748,7 +1881,7 @@ static SolveFn solve_kernel_for(int n) {
 using SolveBatchFn = void (*)(const MPArgs *, const int64_t *, int32_t, int32_t, unsigned *, int, int);
 static SolveBatchFn solve_batched_kernel_for(int n) {
     switch ((n + 7) / 8) {
-    case 1: return mp_solve_batched_kernel<8>;
+    case 1: return n <= 4 ? mp_solve_batched_kernel<4> : mp_solve_batched_kernel<8>;
     case 2: return mp_solve_batched_kernel<16>;
     case 3: return mp_solve_batched_kernel<24>;
     case 4: return mp_solve_batched_kernel<32>;
@@ -1778,10 +1911,10 @@ struct MPLaunch {
 static vmat_status mp_set_attributes() {
     static bool attr = false;
     if (attr) return VMAT_OK;
-    for (int q = 1; q <= MP_NMAX / 8; ++q) {
-        VMAT_CUDA(cudaFuncSetAttribute(solve_kernel_for(8 * q), cudaFuncAttributeMaxDynamicSharedMemorySize,
+    for (int n : {4, 8, 16, 24, 32, 40, 48, 56, 64, 72, 80, 88, 96}) { // every kernel
+        VMAT_CUDA(cudaFuncSetAttribute(solve_kernel_for(n), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        MP_SMEM_LIMIT));
-        VMAT_CUDA(cudaFuncSetAttribute(solve_batched_kernel_for(8 * q), cudaFuncAttributeMaxDynamicSharedMemorySize,
+        VMAT_CUDA(cudaFuncSetAttribute(solve_batched_kernel_for(n), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        MP_SMEM_LIMIT));
     }
     VMAT_CUDA(cudaFuncSetAttribute(mp_iter_ldg_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, MP_SMEM_LIMIT));
@@ -1805,9 +1938,10 @@ static vmat_status mp_configure(int32_t V, int32_t n_ap, const DeviceCtx *ctx, M
     if (L->persistent) VMAT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, L->fn, MP_THREADS, L->smem));
     else VMAT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, mp_iter_ldg_kernel, MP_THREADS, L->smem));
     if (bps < 1) return set_error(VMAT_ECUDA, "mp_bb_solve: the solver kernel does not fit on an SM");
-    // every CTA of the persistent grid must be resident at once (grid barriers)
+    // every CTA of the persistent grid must be resident at once (they wait for one another)
     L->P = (int)std::max<int64_t>(1, std::min<int64_t>(L->persistent ? (n_wtiles + MP_NW - 1) / MP_NW : n_tiles,
                                                         (int64_t)ctx->n_sm * bps));
+    if (L->persistent) L->P = std::min(L->P, mp_cta_cap(solve_nmax(n_ap)));
     L->Pc = std::max(1, std::min<int>(n_tiles, ctx->n_sm * 4));
     return VMAT_OK;
 }
@@ -1815,15 +1949,33 @@ static vmat_status mp_configure(int32_t V, int32_t n_ap, const DeviceCtx *ctx, M
 // Upper bound on co-resident CTAs of MP_THREADS threads (2048 threads per SM).
 static int mp_p_max(const DeviceCtx *ctx) { return ctx->n_sm * (2048 / MP_THREADS); }
 
-static size_t mp_ws_bytes(int n_cap, int p_max) {
-    return 256 + (size_t)(n_cap + 1) * sizeof(double) + (size_t)n_cap * (sizeof(double) + sizeof(float)) +
-           2 * (size_t)p_max * (n_cap + 1) * sizeof(double) + (size_t)p_max * sizeof(double) + 256;
+// Slots and results of the persistent solvers' exchange; the fallback solver's [P][n + 1]
+// partials take the slots' place.
+static int32_t mp_rstride(int n_cap) { return (n_cap + 2 + 7) & ~7; } // whole 128-byte lines
+static size_t mp_exchange_bytes(int n_cap, int p_max) {
+    return ((size_t)p_max * (n_cap + 1) + (size_t)RES_COPIES * mp_rstride(n_cap)) * sizeof(ulonglong2);
 }
+
+static size_t mp_ws_bytes(int n_cap, int p_max) {
+    return 256 + mp_exchange_bytes(n_cap, p_max) + (size_t)(n_cap + 1) * sizeof(double) +
+           (size_t)n_cap * (sizeof(double) + sizeof(float)) + (size_t)p_max * sizeof(double) + 256;
+}
+
+// What has to be zero before the first solve on a workspace: the state word, the tag, the
+// exchange's words.
+static size_t mp_zero_bytes(int n_cap, int p_max) { return 256 + mp_exchange_bytes(n_cap, p_max); }
 
 size_t mp_workspace_bytes(int32_t n_cap) {
     DeviceCtx *ctx;
     if (device_ctx(&ctx) != VMAT_OK) return 0;
     return mp_ws_bytes(n_cap, mp_p_max(ctx));
+}
+
+vmat_status mp_workspace_clear(void *ws, int32_t n_cap, cudaStream_t s) {
+    DeviceCtx *ctx;
+    VMAT_TRY(device_ctx(&ctx));
+    VMAT_CUDA(cudaMemsetAsync(ws, 0, mp_zero_bytes(n_cap, mp_p_max(ctx)), s));
+    return VMAT_OK;
 }
 
 static void mp_fill_args(MPArgs &a, void *ws, int n_cap, int p_max, const float *DA, int64_t wstride, int32_t V,
@@ -1832,14 +1984,15 @@ static void mp_fill_args(MPArgs &a, void *ws, int n_cap, int p_max, const float 
                          const MPLaunch &L, const DeviceCtx *ctx) {
     char *p = static_cast<char *>(ws);
     a.st = reinterpret_cast<BBState *>(p);
-    a.bar_count = reinterpret_cast<unsigned *>(p + 192);
-    a.bar_gen = reinterpret_cast<unsigned *>(p + 224);
-    a.epoch_snap = reinterpret_cast<unsigned *>(p + 240);
+    a.tag = reinterpret_cast<unsigned *>(p + 192);
     p += 256;
-    a.G = reinterpret_cast<double *>(p); // [n + 1]: G, then F in the persistent solver
+    a.slots = reinterpret_cast<ulonglong2 *>(p);
+    a.res = a.slots + (size_t)p_max * (n_cap + 1);
+    a.rstride = mp_rstride(n_cap);
+    a.part = reinterpret_cast<double *>(p);
+    a.G = reinterpret_cast<double *>(p + mp_exchange_bytes(n_cap, p_max)); // [n + 1]
     a.Gprev = a.G + n_cap + 1;
-    a.part = a.Gprev + n_cap;
-    a.cpart = a.part + 2 * (size_t)p_max * (n_cap + 1);
+    a.cpart = a.Gprev + n_cap;
     a.yprev = reinterpret_cast<float *>(a.cpart + p_max);
     a.DA = DA;
     a.wstride = wstride;
@@ -1872,8 +2025,6 @@ static void mp_fill_args(MPArgs &a, void *ws, int n_cap, int p_max, const float 
 }
 
 static vmat_status mp_launch_persistent(MPArgs &a, const MPLaunch &L, cudaStream_t s) {
-    mp_init_kernel<<<1, MP_THREADS, 0, s>>>(a);
-    VMAT_LAUNCH_CHECK();
     int st_arg = L.stages, l2_arg = L.keep_in_l2;
     void *args[] = {&a, &st_arg, &l2_arg};
     VMAT_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(L.fn), dim3(L.P), dim3(MP_THREADS), args,
@@ -1950,7 +2101,8 @@ vmat_status mp_batched_grid(int32_t n, int32_t n_plans, int32_t *grid, int32_t *
     int bps = 0;
     VMAT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, solve_batched_kernel_for(n), MP_THREADS, sm));
     if (bps < 1) return set_error(VMAT_ECUDA, "batched master problem: kernel does not fit on an SM");
-    const int64_t P = (int64_t)ctx->n_sm * bps; // every CTA resident at once (grid barriers)
+    // every CTA resident at once (they wait for one another)
+    const int64_t P = std::min<int64_t>((int64_t)ctx->n_sm * bps, mp_cta_cap(solve_nmax(n)));
     if (P < n_plans) return set_error(VMAT_EUNSUPPORTED, "batched master problem: more plans than resident CTAs");
     *grid = (int32_t)P;
     *stages = st;
@@ -2009,6 +2161,7 @@ vmat_status mp_bb_impl(const float *DA, int32_t V, int32_t n_ap, int64_t ld, con
     if (!host_st) VMAT_CUDA(cudaMallocHost(&host_st, sizeof(BBState)));
 
     if (L.persistent) {
+        VMAT_CUDA(cudaMemsetAsync(ws.ptr, 0, mp_zero_bytes(n_ap, p_max), s));
         VMAT_TRY(mp_launch_persistent(a, L, s));
         VMAT_CUDA(cudaMemcpyAsync(host_st, a.st, sizeof(BBState), cudaMemcpyDeviceToHost, s));
         VMAT_CUDA(cudaStreamSynchronize(s));
