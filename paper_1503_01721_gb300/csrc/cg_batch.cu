@@ -349,7 +349,7 @@ static vmat_status make_batch(Batch &b, int32_t n_plans, const vmat_plan_desc *p
         BPlan &p = b.P[i];
         const Ddc &h = *p.h;
         const bool fp8 = h.dtype == VMAT_FP8E4M3;
-        spmv[i] = SpmvPlan{h.Dt.rowptr, h.Dt.col, h.Dt.val, p.g_full, p.pi, fp8 ? h.scale : nullptr, nullptr,
+        spmv[i] = SpmvPlan{h.Dt.rowptr, h.Dt.col, h.Dt.val, h.Dt.strm, h.Dt.sptr, p.g_full, p.pi, fp8 ? h.scale : nullptr, nullptr,
                            RowMask{nullptr, p.win, p.bpc, p.mlc.n_cols}, p.ctl, h.Dt.n_rows};
         PricePlan &q = price[i];
         VMAT_TRY(pricing_geom(&p.mlc, &q.g));

@@ -406,8 +406,10 @@ extern "C" vmat_status cg_plan(vmat_ddc hd, const vmat_mlc *mlc, const vmat_voxe
     if (refine) {
         hf.dtype = VMAT_F32;
         hf.D.val = h.D_val_f32;
+        hf.D.strm = nullptr; // the packed stream and the CP-major copy hold the stored values
+        hf.D.sptr = nullptr;
         hf.scale = nullptr;
-        hf.cpm_loc = nullptr; // the CP-major copy holds the stored values
+        hf.cpm_loc = nullptr;
         hf.cpm_val = nullptr;
         hf.cpm_base = nullptr;
     }

@@ -78,6 +78,8 @@ void Ddc::free_all() {
         f(m->col16);
         f(m->cbase);
         f(m->cptr);
+        f(m->strm);
+        f(m->sptr);
         *m = CsrMat();
     }
     f(act_vox);

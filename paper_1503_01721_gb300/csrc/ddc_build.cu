@@ -681,7 +681,104 @@ __global__ void fill_index16(const int64_t *__restrict__ rowptr, const int32_t *
     }
 }
 
+// Records of STRM_ENTRIES entries per row (the last one ragged).
+__global__ void record_counts(const int64_t *__restrict__ rowptr, int32_t n_rows, int32_t *cnt) {
+    for (int32_t r = blockIdx.x * blockDim.x + threadIdx.x; r < n_rows; r += gridDim.x * blockDim.x)
+        cnt[r] = (int32_t)((rowptr[r + 1] - rowptr[r] + STRM_ENTRIES - 1) / STRM_ENTRIES);
+}
+
+__global__ void narrow_offsets(const int64_t *in, int64_t n, int32_t *out) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        out[i] = (int32_t)in[i];
+}
+
+// A warp per row writes its records; far[0] counts the 32-entry chunks whose columns span
+// 65,536 or more.
+template <typename V> struct Vec4 { V v[4]; };
+template <typename V>
+__global__ void fill_stream(const int64_t *__restrict__ rowptr, const int32_t *__restrict__ col,
+                            const V *__restrict__ val, const int32_t *__restrict__ sptr, int32_t n_rows,
+                            unsigned char *__restrict__ strm, unsigned long long *far) {
+    const int lane = threadIdx.x & 31;
+    unsigned long long n_far = 0;
+    for (int32_t r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < n_rows; r += (gridDim.x * blockDim.x) >> 5) {
+        const int64_t s = rowptr[r], e = rowptr[r + 1];
+        unsigned char *rec = strm + (int64_t)sptr[r] * strm_record_bytes(sizeof(V));
+        for (int64_t b = s; b < e; b += STRM_ENTRIES, rec += strm_record_bytes(sizeof(V))) {
+            int32_t my_base = 0;
+            uint32_t off[4];
+            Vec4<V> v;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int64_t i = b + 32 * u + lane;
+                const bool in = i < e;
+                const int32_t c = in ? col[i] : 0;
+                v.v[u] = in ? val[i] : V(0);
+                int32_t base = __shfl_sync(0xffffffffu, c, 0); // rows are sorted: the chunk's smallest column
+                const uint32_t d = in ? (uint32_t)(c - base) : 0u;
+                if (__any_sync(0xffffffffu, d > 65535u)) {
+                    base = -1;
+                    ++n_far;
+                }
+                off[u] = base < 0 ? 0u : d;
+                if (lane == u) my_base = base;
+            }
+            if (lane < 4) reinterpret_cast<int32_t *>(rec)[lane] = my_base;
+            reinterpret_cast<uint2 *>(rec + 16)[lane] = make_uint2(off[0] | (off[1] << 16), off[2] | (off[3] << 16));
+            unsigned char *vp = rec + 16 + STRM_ENTRIES * 2 + lane * 4 * sizeof(V);
+            if (sizeof(V) == 4) *reinterpret_cast<uint4 *>(vp) = *reinterpret_cast<const uint4 *>(&v);
+            else if (sizeof(V) == 2) *reinterpret_cast<uint2 *>(vp) = *reinterpret_cast<const uint2 *>(&v);
+            else *reinterpret_cast<uint32_t *>(vp) = *reinterpret_cast<const uint32_t *>(&v);
+        }
+    }
+    if (lane == 0 && n_far) atomicAdd(far, n_far);
+}
+
 } // namespace
+
+vmat_status csr_build_stream(CsrMat &m, int vb, int n_sm, cudaStream_t s) {
+    if (m.n_rows <= 0 || m.nnz <= 0) return VMAT_OK;
+    DevBuf b_cnt, b_ptr, b_sptr, b_strm, b_far;
+    const auto skip = [] { // no room: the configurations read col and val
+        cudaGetLastError();
+        return VMAT_OK;
+    };
+    if (b_cnt.alloc((size_t)m.n_rows * 4) != cudaSuccess || b_ptr.alloc((size_t)(m.n_rows + 1) * 8) != cudaSuccess ||
+        b_sptr.alloc((size_t)(m.n_rows + 1) * 4) != cudaSuccess || b_far.alloc(8) != cudaSuccess)
+        return skip();
+    record_counts<<<grid_for(m.n_rows, n_sm), BUILD_THREADS, 0, s>>>(m.rowptr, m.n_rows, (int32_t *)b_cnt.p);
+    VMAT_LAUNCH_CHECK();
+    VMAT_TRY(scan_counts((int32_t *)b_cnt.p, (int64_t *)b_ptr.p, m.n_rows, s));
+    int64_t n_rec = 0;
+    VMAT_CUDA(cudaMemcpyAsync(&n_rec, (int64_t *)b_ptr.p + m.n_rows, 8, cudaMemcpyDeviceToHost, s));
+    VMAT_CUDA(cudaMemsetAsync(b_far.p, 0, 8, s));
+    VMAT_CUDA(cudaStreamSynchronize(s));
+    if (n_rec > INT32_MAX) return VMAT_OK;
+    // rows of a few entries pad most of a record: such a matrix would read more, not less
+    if ((double)n_rec * strm_record_bytes(vb) > (double)m.nnz * (vb + 4)) return VMAT_OK;
+    if (b_strm.alloc((size_t)n_rec * strm_record_bytes(vb)) != cudaSuccess) return skip();
+    narrow_offsets<<<grid_for(m.n_rows + 1, n_sm), BUILD_THREADS, 0, s>>>((int64_t *)b_ptr.p, m.n_rows + 1,
+                                                                         (int32_t *)b_sptr.p);
+    VMAT_LAUNCH_CHECK();
+    const int g = grid_for((int64_t)m.n_rows * 32, n_sm);
+    auto *far = (unsigned long long *)b_far.p;
+    auto *strm = (unsigned char *)b_strm.p;
+    const int32_t *sp = (const int32_t *)b_sptr.p;
+    if (vb == 4)
+        fill_stream<uint32_t><<<g, BUILD_THREADS, 0, s>>>(m.rowptr, m.col, (const uint32_t *)m.val, sp, m.n_rows, strm, far);
+    else if (vb == 2)
+        fill_stream<uint16_t><<<g, BUILD_THREADS, 0, s>>>(m.rowptr, m.col, (const uint16_t *)m.val, sp, m.n_rows, strm, far);
+    else
+        fill_stream<uint8_t><<<g, BUILD_THREADS, 0, s>>>(m.rowptr, m.col, (const uint8_t *)m.val, sp, m.n_rows, strm, far);
+    VMAT_LAUNCH_CHECK();
+    unsigned long long n_far = 0;
+    VMAT_CUDA(cudaMemcpyAsync(&n_far, far, 8, cudaMemcpyDeviceToHost, s));
+    VMAT_CUDA(cudaStreamSynchronize(s));
+    if (n_far * 16 > (unsigned long long)n_rec * (STRM_ENTRIES / 32)) return VMAT_OK;
+    m.strm = (unsigned char *)b_strm.release();
+    m.sptr = (int32_t *)b_sptr.release();
+    return VMAT_OK;
+}
 
 vmat_status csr_build_index16(CsrMat &m, int n_sm, cudaStream_t s) {
     if (m.n_rows <= 0 || m.nnz <= 0) return VMAT_OK;
@@ -930,6 +1027,7 @@ extern "C" vmat_status ddc_build(vmat_ddc hd, const vmat_build_opts *opts_in, vo
         m.row_ids = nullptr;
         m.max_row = max_row_t;
         if (opts.index16) VMAT_TRY(csr_build_index16(m, n_sm, s));
+        if (opts.autotune || spmv_config_stream(cfg_dt)) VMAT_TRY(csr_build_stream(m, vb, n_sm, s));
         VMAT_TRY(spmv_prepare_tiles(m, cfg_dt, s));
         h->built_Dt = true;
     }
@@ -958,6 +1056,7 @@ extern "C" vmat_status ddc_build(vmat_ddc hd, const vmat_build_opts *opts_in, vo
         m.row_ids = h->act_vox;
         m.max_row = max_row_d;
         if (opts.index16) VMAT_TRY(csr_build_index16(m, n_sm, s));
+        if (opts.autotune || spmv_config_stream(cfg)) VMAT_TRY(csr_build_stream(m, vb, n_sm, s));
         VMAT_TRY(spmv_prepare_tiles(m, cfg, s));
         h->built_D = true;
     }

@@ -104,6 +104,10 @@ struct CsrMat {
     int32_t *cbase = nullptr;    // [n_chunks]
     int64_t *cptr = nullptr;     // [n_rows + 1] first chunk of each row
     int64_t n_chunks = 0;
+    // The matrix once more as a packed stream for the consecutive-lane configurations (null:
+    // they read col and val): see csr_build_stream.
+    unsigned char *strm = nullptr; // [strm_recs] records
+    int32_t *sptr = nullptr;       // [n_rows + 1] first record of each row
     // tiles
     int cfg = 0;                 // tile configuration index
     int32_t tile = 0;            // nonzeros per tile
@@ -243,6 +247,20 @@ vmat_status spmv_prepare_tiles(CsrMat &m, int cfg, cudaStream_t s);
 vmat_status ddc_window_config(Ddc &h, int32_t n_cols, int32_t nseg, cudaStream_t s, int *cfg);
 // Does configuration cfg read the 16-bit column index (and so need m.col16)?
 bool spmv_config_index16(int cfg);
+// Packed stream (csr_build_stream): every row in records of STRM_ENTRIES consecutive entries,
+//     int32 base[4] | uint16 offset[32][4] | value[32][4]
+// entry 32 u + l of a record in lane l's place u: its column is base[u] + offset[l][u], the
+// first column of its 32 entries plus a 16-bit offset.  base[u] = -1: those 32 entries span
+// 65,536 columns or more, and their columns are read from col.  The last record of a row is
+// padded with zeros (never read as entries).  A lane reads its four offsets and its four
+// values with one load each, and a gather of x still covers 32 consecutive entries.
+constexpr int STRM_ENTRIES = 128;
+__host__ __device__ constexpr int strm_record_bytes(int vb) { return 16 + STRM_ENTRIES * (2 + vb); }
+// Is configuration cfg one that reads the packed stream when the matrix holds it?
+bool spmv_config_stream(int cfg);
+// Builds m.strm / m.sptr from m.col and m.val (vb bytes per value).  VMAT_OK without it when
+// memory is short or when more than 1/16 of the 32-entry chunks span 65,536 columns.
+vmat_status csr_build_stream(CsrMat &m, int vb, int n_sm, cudaStream_t s);
 // Builds m.col16 / cbase / cptr when every chunk fits 16 bits (else leaves them null).
 vmat_status csr_build_index16(CsrMat &m, int n_sm, cudaStream_t s);
 int spmv_n_configs();
@@ -271,6 +289,8 @@ struct SpmvPlan { // one plan's matrix and vectors in a batched warp-row SpMV
     const int64_t *rowptr;
     const int32_t *col;
     const void *val;
+    const unsigned char *strm; // packed stream of the matrix, or null
+    const int32_t *sptr;
     const float *x;
     float *y;
     const float *row_scale; // or null

@@ -393,6 +393,8 @@ struct RowParams {
     int32_t n_rows;
     int64_t stride; // rows between a warp's consecutive rows (<= the launch's warps; warps past it idle)
     const int32_t *skip; // when non-null and set, the kernel does nothing
+    const unsigned char *strm; // packed stream (spmv_warp_row_x_kernel)
+    const int32_t *sptr;
     const uint16_t *col16; // 16-bit column index (configurations that read it)
     const int32_t *cbase;
     const int64_t *cptr;
@@ -514,6 +516,116 @@ __device__ __forceinline__ float warp_row_sum_z(const int64_t *__restrict__ rowp
     return sum;
 }
 
+// The consecutive-lane row sum from the packed stream (records of 128 entries, csr_build_stream):
+// the same products added in the same order as warp_row_sum_c, so the same bits.  A lane
+// takes its four offsets and its four values with one load each: a record is 784, 528 or 400
+// contiguous bytes in FP32, BF16 or FP8 and three loads, where the CSR's 128 entries are
+// 1,024, 768 or 640 bytes and eight.
+//
+// What bounds it: the gathers of x in L1, about two cycles per 128-byte line touched (3.5 lines per
+// 32 entries of a beamlet row in brick order): the times hardly follow the bytes.  So many
+// warps are kept resident (32 registers, 64 warps per SM).  484M nonzeros (128 x 128 x 96
+// voxels, 90 CPs, brick order), the CSR's fastest configuration -> this one: D^T g FP32 0.696 ->
+// 0.620 ms, BF16 0.615 -> 0.520, FP8 0.534 -> 0.491; D x 0.728 -> 0.703, 0.689 -> 0.663, 0.695
+// -> 0.625.  Slower: the next record in flight in registers (48 registers: 0.693 ms FP32), two
+// records at once, and prefetching the next records into L2 (0.678 ms).
+// (The values stay as loaded until their products: a conversion would wait for the load.)
+template <typename VT> struct RawVals;
+template <> struct RawVals<float> {
+    float4 r;
+    __device__ __forceinline__ void load(const void *q, int lane, uint64_t pol) {
+        r = ldg_stream_f4(static_cast<const float4 *>(q) + lane, pol);
+    }
+    __device__ __forceinline__ void get(float v[4]) const {
+        v[0] = r.x;
+        v[1] = r.y;
+        v[2] = r.z;
+        v[3] = r.w;
+    }
+};
+template <> struct RawVals<__nv_bfloat16> {
+    uint2 r;
+    __device__ __forceinline__ void load(const void *q, int lane, uint64_t pol) {
+        r = ldg_stream_u2(static_cast<const uint2 *>(q) + lane, pol);
+    }
+    __device__ __forceinline__ void get(float v[4]) const {
+        v[0] = __uint_as_float(r.x << 16);
+        v[1] = __uint_as_float(r.x & 0xffff0000u);
+        v[2] = __uint_as_float(r.y << 16);
+        v[3] = __uint_as_float(r.y & 0xffff0000u);
+    }
+};
+template <> struct RawVals<__nv_fp8_e4m3> {
+    uint32_t r;
+    __device__ __forceinline__ void load(const void *q, int lane, uint64_t pol) {
+        r = ldg_stream_u1(static_cast<const uint32_t *>(q) + lane, pol);
+    }
+    __device__ __forceinline__ void get(float v[4]) const {
+        __half2_raw a = __nv_cvt_fp8x2_to_halfraw2((__nv_fp8x2_storage_t)(r & 0xffffu), __NV_E4M3);
+        __half2_raw b = __nv_cvt_fp8x2_to_halfraw2((__nv_fp8x2_storage_t)(r >> 16), __NV_E4M3);
+        const float2 fa = __half22float2(*reinterpret_cast<__half2 *>(&a));
+        const float2 fb = __half22float2(*reinterpret_cast<__half2 *>(&b));
+        v[0] = fa.x;
+        v[1] = fa.y;
+        v[2] = fb.x;
+        v[3] = fb.y;
+    }
+};
+template <typename VT> struct StreamRec {
+    RawVals<VT> v;
+    uint2 o;
+    int4 b;
+    __device__ __forceinline__ void load(const unsigned char *q, int lane, uint64_t pol) {
+        b = ldg_stream_i4(q, pol);
+        o = ldg_stream_u2(q + 16 + lane * 8, pol);
+        v.load(q + 16 + STRM_ENTRIES * 2, lane, pol);
+    }
+};
+// acc[u] += value * x over one record; left: the row's entries from the record on (> 0), col: their columns.
+template <typename VT>
+__device__ __forceinline__ void record_products(const StreamRec<VT> &q, const int32_t *__restrict__ col, int left,
+                                                const float *__restrict__ x, int lane, float acc[4]) {
+    const int32_t bs[4] = {q.b.x, q.b.y, q.b.z, q.b.w};
+    int32_t j[4] = {bs[0] + (int32_t)(q.o.x & 0xffffu), bs[1] + (int32_t)(q.o.x >> 16),
+                    bs[2] + (int32_t)(q.o.y & 0xffffu), bs[3] + (int32_t)(q.o.y >> 16)};
+    if ((bs[0] | bs[1] | bs[2] | bs[3]) < 0) { // a chunk that spans 65,536 columns or more
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (bs[u] < 0 && 32 * u + lane < left) j[u] = __ldg(col + 32 * u + lane);
+    }
+    float v[4];
+    q.v.get(v);
+    if (left >= STRM_ENTRIES) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc[u] = fmaf(v[u], __ldg(x + j[u]), acc[u]);
+    } else {
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (32 * u + lane < left) acc[u] = fmaf(v[u], __ldg(x + j[u]), acc[u]);
+    }
+}
+template <typename VT>
+__device__ __forceinline__ float warp_row_sum_x(const int64_t *__restrict__ rowptr, const int32_t *__restrict__ col,
+                                                const unsigned char *__restrict__ strm,
+                                                const int32_t *__restrict__ sptr, const float *__restrict__ x,
+                                                int64_t r, int lane, uint64_t pol) {
+    constexpr int REC = strm_record_bytes((int)sizeof(VT));
+    const int64_t s = __ldg(rowptr + r);
+    int n = (int)(__ldg(rowptr + r + 1) - s);
+    const unsigned char *rec = strm + (int64_t)__ldg(sptr + r) * REC;
+    const int32_t *c = col + s;
+    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+    for (; n > 0; n -= STRM_ENTRIES, rec += REC, c += STRM_ENTRIES) {
+        StreamRec<VT> q;
+        q.load(rec, lane, pol);
+        record_products<VT>(q, c, n, x, lane, acc);
+    }
+    float sum = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, d);
+    return sum;
+}
+
 // The rows of a warp-row launch, passed to f in order.  Without a list: rows
 // warp0, warp0 + stride, ... that the mask keeps.  With the window list (mask.woff):
 // list items in runs of WIN_RUN consecutive items, run warp0, warp0 + stride, ...; the
@@ -557,6 +669,22 @@ __global__ void __launch_bounds__(THREADS) spmv_warp_row_z_kernel(RowParams p) {
     const uint64_t pol = l2_evict_first_policy();
     for_rows(p, warp0, [&](int64_t r) {
         float sum = warp_row_sum_z<UNROLL, VT>(p.rowptr, p.cptr, p.cbase, p.col16, p.val, p.x, r, lane, pol);
+        if (lane == 0) {
+            if (p.row_scale) sum *= p.row_scale[r];
+            p.y[p.row_ids ? p.row_ids[r] : r] = sum;
+        }
+    });
+}
+
+template <int THREADS, int CTAS, typename VT>
+__global__ void __launch_bounds__(THREADS, CTAS) spmv_warp_row_x_kernel(RowParams p) {
+    if (p.skip && *p.skip) return;
+    const int lane = threadIdx.x & 31;
+    const int64_t warp0 = ((int64_t)blockIdx.x * THREADS + threadIdx.x) >> 5;
+    if (warp0 >= p.stride) return; // warp-uniform
+    const uint64_t pol = l2_evict_first_policy();
+    for_rows(p, warp0, [&](int64_t r) {
+        float sum = warp_row_sum_x<VT>(p.rowptr, p.col, p.strm, p.sptr, p.x, r, lane, pol);
         if (lane == 0) {
             if (p.row_scale) sum *= p.row_scale[r];
             p.y[p.row_ids ? p.row_ids[r] : r] = sum;
@@ -629,8 +757,9 @@ __global__ void __launch_bounds__(THREADS)
         if (skip) continue;
         const int64_t r = gr - lo;
         if (!row_needed(P.mask, r)) continue;
-        float sum = CONSEC ? warp_row_sum_c<UNROLL, VT>(P.rowptr, P.col, P.val, P.x, r, lane, pol)
-                           : warp_row_sum<UNROLL, VT>(P.rowptr, P.col, P.val, P.x, r, lane, pol);
+        float sum = !CONSEC  ? warp_row_sum<UNROLL, VT>(P.rowptr, P.col, P.val, P.x, r, lane, pol)
+                    : P.strm ? warp_row_sum_x<VT>(P.rowptr, P.col, P.strm, P.sptr, P.x, r, lane, pol)
+                             : warp_row_sum_c<UNROLL, VT>(P.rowptr, P.col, P.val, P.x, r, lane, pol);
         if (lane == 0) {
             if (P.row_scale) sum *= P.row_scale[r];
             P.y[P.row_ids ? P.row_ids[r] : r] = sum;
@@ -770,6 +899,16 @@ template <typename VT> RowFn row_kernel_for(int cfg) {
     }
 }
 
+// The stream's kernel for a consecutive-lane configuration: 256 threads with 8 or 6 CTAs per
+// SM (32 or 40 registers), 512 with 4.  The autotuner times them as it times the others.
+template <typename VT> RowFn stream_kernel_for(int cfg) {
+    switch (cfg) {
+    case 9: return spmv_warp_row_x_kernel<256, 8, VT>;
+    case 10: return spmv_warp_row_x_kernel<256, 6, VT>;
+    default: return spmv_warp_row_x_kernel<512, 4, VT>;
+    }
+}
+
 template <typename VT> int smem_for(int cfg) {
     switch (cfg) {
     case 0: return TileShape<256, 16, 2, VT>::SMEM;
@@ -783,7 +922,8 @@ template <typename VT> int smem_for(int cfg) {
 struct Launch {
     TileFn tile = nullptr;
     RowFn row = nullptr;
-    int threads = 0, smem = 0, blocks_per_sm = 0;
+    RowFn strm = nullptr; // the same configuration reading the packed stream
+    int threads = 0, smem = 0, blocks_per_sm = 0, blocks_strm = 0;
 };
 
 template <typename VT> static void pick(int cfg, Launch &n) {
@@ -792,6 +932,7 @@ template <typename VT> static void pick(int cfg, Launch &n) {
         n.smem = smem_for<VT>(cfg);
     } else {
         n.row = row_kernel_for<VT>(cfg);
+        if (kCfgs[cfg].family == 2) n.strm = stream_kernel_for<VT>(cfg);
         n.smem = 0;
     }
 }
@@ -816,6 +957,7 @@ static vmat_status launch_info(vmat_dtype dt, int cfg, Launch *out) {
         VMAT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n.blocks_per_sm, n.tile, n.threads, n.smem));
     } else {
         VMAT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n.blocks_per_sm, n.row, n.threads, 0));
+        if (n.strm) VMAT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n.blocks_strm, n.strm, n.threads, 0));
     }
     if (n.blocks_per_sm < 1) return set_error(VMAT_ECUDA, "spmv: configuration %d does not fit on an SM", cfg);
     L = n;
@@ -825,6 +967,7 @@ static vmat_status launch_info(vmat_dtype dt, int cfg, Launch *out) {
 }
 
 int spmv_n_configs() { return N_CFG; }
+bool spmv_config_stream(int cfg) { return cfg >= 0 && cfg < N_CFG && kCfgs[cfg].family == 2; }
 bool spmv_config_index16(int cfg) { return cfg >= 0 && cfg < N_CFG && kCfgs[cfg].family == 3; }
 int spmv_default_config() { return 4; }
 int32_t spmv_config_tile(int cfg) { return kCfgs[cfg].family == 0 ? kCfgs[cfg].threads * kCfgs[cfg].e : 0; }
@@ -885,6 +1028,9 @@ vmat_status spmv_run(const Ddc &h, const CsrMat &m, const float *x, float *y, co
         p.mask = mask;
         p.n_rows = m.n_rows;
         p.skip = skip;
+        const bool strm = L.strm && m.strm && L.blocks_strm > 0;
+        p.strm = m.strm;
+        p.sptr = m.sptr;
         p.col16 = m.col16;
         p.cbase = m.cbase;
         p.cptr = m.cptr;
@@ -892,10 +1038,11 @@ vmat_status spmv_run(const Ddc &h, const CsrMat &m, const float *x, float *y, co
             return set_error(VMAT_ESTATE, "spmv: configuration %d needs the 16-bit column index", m.cfg);
         const int64_t warps = std::max<int64_t>(1, m.n_rows);
         const int64_t want = (warps * 32 + L.threads - 1) / L.threads;
-        const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)ctx->n_sm * L.blocks_per_sm));
+        const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)ctx->n_sm * (strm ? L.blocks_strm
+                                                                                                             : L.blocks_per_sm)));
         const int64_t n_warps = (int64_t)grid * L.threads / 32;
         p.stride = mask.win && !mask.woff ? coprime_stride(n_warps, &mask.n_cols, 1) : n_warps;
-        L.row<<<grid, L.threads, 0, s>>>(p);
+        (strm ? L.strm : L.row)<<<grid, L.threads, 0, s>>>(p);
         VMAT_LAUNCH_CHECK();
         return VMAT_OK;
     }
