@@ -65,16 +65,6 @@ __device__ int nearest_occupied(const PricingGeom &g, const uint8_t *occupied, i
     return -1;
 }
 
-// The same search by one thread.
-__device__ int nearest_occupied_seq(const PricingGeom &g, const uint8_t *occupied, int k, int dir) {
-    int a = 0;
-    while (a + 1 < g.n_arcs && g.arc_first[a + 1] <= k) ++a;
-    const int lo = g.arc_first[a], hi = g.arc_first[a + 1];
-    for (int kk = k + dir; kk >= lo && kk < hi; kk += dir)
-        if (occupied[kk]) return kk;
-    return -1;
-}
-
 // Leaf-travel window of MLC row r at CP k (reading R7): each leaf moves at most
 // travel columns per CP step from its position at the nearest occupied CP on each
 // side (kl, kr; -1: none).
@@ -113,9 +103,9 @@ __device__ __forceinline__ void window_prefix(const float *__restrict__ row, int
     }
 }
 
-// Shared memory per warp of the row kernel: the float64 prefix sums and their
-// float32 roundings, n_cols + 1 of each.
-__host__ __device__ constexpr size_t row_smem_stride(int n_cols) { return (((size_t)(n_cols + 1) * 12) + 15) & ~15; }
+// Shared memory per warp of the row kernel: the float64 prefix sums, their float32
+// roundings and each left leaf's best float32 value, n_cols + 1 of each.
+__host__ __device__ constexpr size_t row_smem_stride(int n_cols) { return (((size_t)(n_cols + 1) * 16) + 15) & ~15; }
 
 // Best opening of MLC row r of CP k (one warp; ws: row_smem_stride(n_cols) bytes of
 // shared memory for this warp).  Writes the row's entry gw of rb_*.
@@ -128,7 +118,9 @@ __host__ __device__ constexpr size_t row_smem_stride(int n_cols) { return (((siz
 // two roundings of P to float32, one float32 and one float64 subtraction, each at
 // most 2^-24 or 2^-53 relative, with a factor 4 to spare).  The pairs that attain
 // the float64 maximum are always among them, so the choice, ties included, is the
-// one the exhaustive float64 search makes.
+// one the exhaustive float64 search makes.  The first pass keeps each left leaf's float32
+// maximum, and the second visits only the left leaves whose maximum reaches the threshold,
+// a few of a row's (it used to walk every pair again, half of the search's time).
 __device__ __forceinline__ void price_row_warp(const PricingGeom &g, const float *__restrict__ pi,
                                                const uint8_t *__restrict__ occupied, const int16_t *__restrict__ leaves,
                                                int64_t gw, unsigned char *ws, double *rb_v, int16_t *rb_lr,
@@ -139,6 +131,7 @@ __device__ __forceinline__ void price_row_warp(const PricingGeom &g, const float
     const int N = g.n_cols;
     double *P = reinterpret_cast<double *>(ws);
     float *P32 = reinterpret_cast<float *>(ws + (size_t)(N + 1) * 8);
+    float *best32 = P32 + (N + 1); // a lane reads the entries it wrote
     const int kl = nearest_occupied(g, occupied, k, -1, lane), kr = nearest_occupied(g, occupied, k, 1, lane);
     const RowWindow win = row_window(g, leaves, k, r, kl, kr);
     const int Lmin = win.Lmin, Lmax = win.Lmax, Rmin = win.Rmin, Rmax = win.Rmax;
@@ -161,7 +154,18 @@ __device__ __forceinline__ void price_row_warp(const PricingGeom &g, const float
     float m32 = -INFINITY;
     for (int L = Lmin + lane; L <= Lmax; L += 32) {
         const float pl = P32[L];
-        for (int R = max(L, Rmin); R <= Rmax; ++R) m32 = fmaxf(m32, P32[R] - pl);
+        // four maxima: a chain of one per pair would wait for the one before
+        float m[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+        int R = max(L, Rmin);
+        // (a price that is not a number makes every later sum one: its pairs stay candidates)
+        const bool nan = R <= Rmax && (isnan(pl) || isnan(P32[Rmax]));
+        for (; R + 3 <= Rmax; R += 4)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) m[q] = fmaxf(m[q], P32[R + q] - pl);
+        for (; R <= Rmax; ++R) m[0] = fmaxf(m[0], P32[R] - pl);
+        const float ml = fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3]));
+        best32[L] = nan ? INFINITY : ml;
+        m32 = fmaxf(m32, ml);
     }
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) m32 = fmaxf(m32, __shfl_xor_sync(0xffffffffu, m32, d));
@@ -174,6 +178,7 @@ __device__ __forceinline__ void price_row_warp(const PricingGeom &g, const float
     best.key = 0;
     best.w = best.cd = best.L = 0;
     for (int L = Lmin + lane; L <= Lmax; L += 32) {
+        if (best32[L] < thr) continue; // every pair of this left leaf is below the threshold
         const float pl = P32[L];
         const long long bl = __double_as_longlong(P[L]);
         for (int R = max(L, Rmin); R <= Rmax; ++R) {
@@ -221,6 +226,32 @@ __global__ void __launch_bounds__(PR_WARPS * 32)
 
 constexpr int CP_THREADS = 1024;
 
+// Sum of rb_v[i0 .. i0 + n) in order; false when a row has no opening.  The loads of eight
+// rows are issued together: stopping at the first row without an opening made every load
+// wait for the one before (180 CPs of 64 rows: 15 us for the kernel, an L2 access per row).
+__device__ __forceinline__ bool row_best_sum(const double *__restrict__ rb_v, const uint8_t *__restrict__ rb_ok,
+                                             int64_t i0, int n, double *sum) {
+    double price = 0.0;
+    unsigned ok = 1;
+    int r = 0;
+    for (; r + 8 <= n; r += 8) {
+        double v[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            v[q] = rb_v[i0 + r + q];
+            ok &= rb_ok[i0 + r + q] ? 1u : 0u;
+        }
+#pragma unroll
+        for (int q = 0; q < 8; ++q) price = price + v[q];
+    }
+    for (; r < n; ++r) {
+        ok &= rb_ok[i0 + r] ? 1u : 0u;
+        price = price + rb_v[i0 + r];
+    }
+    *sum = price;
+    return ok != 0;
+}
+
 // The CP with the largest price (sum of its row bests, in row order), smallest k
 // on ties, and its leaves (one block).
 __device__ __forceinline__ void price_cps_block(const PricingGeom &g, const uint8_t *__restrict__ occupied,
@@ -236,12 +267,7 @@ __device__ __forceinline__ void price_cps_block(const PricingGeom &g, const uint
     for (int k = threadIdx.x; k < g.K; k += blockDim.x) { // k ascending: a strict > keeps the smallest k
         if (occupied[k]) continue;
         double price = 0.0;
-        bool ok = true;
-        for (int r = 0; r < g.n_rows; ++r) {
-            const int64_t i = (int64_t)k * g.n_rows + r;
-            ok = ok && rb_ok[i];
-            price = price + rb_v[i];
-        }
+        const bool ok = row_best_sum(rb_v, rb_ok, (int64_t)k * g.n_rows, g.n_rows, &price);
         if (ok && (bk < 0 || price > bv)) {
             bv = price;
             bk = k;
@@ -353,19 +379,38 @@ __host__ __device__ constexpr size_t interdig_smem(int N) {
 // float64 in column order, as the definition), for the chain kernels and the row
 // kernel.  FP64 issues at a small fraction of the FP32 rate on this GPU: a row per
 // lane keeps 32 rows' sequential sums in one instruction stream, where a row per
-// warp spends a warp-wide FP64 instruction on every add of one row.
+// warp spends a warp-wide FP64 instruction on every add of one row.  A warp takes 32 rows
+// of one CP, so that it finds the CP's neighbours together (a thread's own search read the
+// occupancy byte by byte), and loads eight prices before it adds them.
 __global__ void window_prefix_kernel(PricingGeom g, const float *__restrict__ pi,
                                        const uint8_t *__restrict__ occupied, const int16_t *__restrict__ leaves,
                                        double *__restrict__ Pall, const int32_t *skip) {
     if (skip && *skip) return;
-    const int N = g.n_cols;
-    for (int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; row < (int64_t)g.K * g.n_rows;
-         row += (int64_t)gridDim.x * blockDim.x) {
-        const int k = (int)(row / g.n_rows), r = (int)(row % g.n_rows);
-        if (occupied[k]) continue;
-        const RowWindow w = row_window(g, leaves, k, r, nearest_occupied_seq(g, occupied, k, -1),
-                                       nearest_occupied_seq(g, occupied, k, 1));
-        window_prefix(pi + row * N, N, w.Lmin, w.Rmax, Pall + row * (N + 1));
+    const int N = g.n_cols, lane = threadIdx.x & 31;
+    const int per = (g.n_rows + 31) / 32; // warps per CP
+    for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < (int64_t)g.K * per;
+         w += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+        const int k = (int)(w / per), r = (int)(w - (int64_t)k * per) * 32 + lane;
+        if (occupied[k]) continue; // warp-uniform
+        const int kl = nearest_occupied(g, occupied, k, -1, lane), kr = nearest_occupied(g, occupied, k, 1, lane);
+        if (r >= g.n_rows) continue;
+        const RowWindow x = row_window(g, leaves, k, r, kl, kr);
+        const int64_t row = (int64_t)k * g.n_rows + r;
+        const float *p = pi + row * N;
+        double *P = Pall + row * (N + 1);
+        double acc = 0.0;
+        P[0] = 0.0;
+        for (int c0 = 0; c0 < N; c0 += 8) {
+            float v[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) v[q] = c0 + q >= x.Lmin && c0 + q < min(x.Rmax, N) ? p[c0 + q] : 0.f;
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+                if (c0 + q < N) {
+                    if (c0 + q >= x.Lmin && c0 + q < x.Rmax) acc = acc + (double)v[q];
+                    P[c0 + q + 1] = acc;
+                }
+        }
     }
 }
 
@@ -779,13 +824,7 @@ __global__ void __launch_bounds__(ID_SEL_THREADS)
         double b = -INFINITY;
         if (!occupied[k]) {
             double price = 0.0;
-            bool ok = true;
-            for (int r = 0; r < g.n_rows; ++r) {
-                const int64_t i = (int64_t)k * g.n_rows + r;
-                ok = ok && rb_ok[i];
-                price = price + rb_v[i];
-            }
-            if (ok) {
+            if (row_best_sum(rb_v, rb_ok, (int64_t)k * g.n_rows, g.n_rows, &price)) {
                 b = price;
                 // nonzero (the low bit only orders the first round, which any order keeps exact)
                 key = order_key(price) | 1ull;
@@ -881,43 +920,76 @@ __global__ void __launch_bounds__(ID_SEL_THREADS)
     if (threadIdx.x == 0) ctl[IDC_N2] = n2;
 }
 
-// The best CP (price desc, smallest k on ties, in k order as the sequential
-// definition: the warp loads 32 CPs at a time and every lane applies the same
-// comparisons in k order) and its leaves, backtracked through the predecessor table
-// its chain stored.
-__global__ void price_pick_interdig_kernel(PricingGeom g, const uint8_t *__restrict__ occupied,
+// The best CP (price desc, smallest k on ties) and its leaves, backtracked through the
+// predecessor table its chain stored.
+constexpr int PICK_THREADS = 1024, PICK_ROWS = 8;
+__host__ __device__ constexpr size_t pick_smem(int N) { return ((size_t)PICK_ROWS * (N + 1) * (N + 1) + 16) * sizeof(int16_t); }
+
+__global__ void __launch_bounds__(PICK_THREADS) price_pick_interdig_kernel(PricingGeom g, const uint8_t *__restrict__ occupied,
                                            const double *cp_val, const uint8_t *cp_ok, const int16_t *pred_all,
                                            int32_t *best_cp, int16_t *best_leaves, double *best_price,
                                            const int32_t *skip) {
     if (skip && *skip) return;
-    const int lane = threadIdx.x;
-    int kb = -1;
-    double v = -INFINITY;
-    for (int base = 0; base < g.K; base += 32) {
-        const int k = base + lane;
-        const bool cand = k < g.K && !occupied[k] && cp_ok[k];
-        const double x = cand ? cp_val[k] : 0.0;
-        const unsigned m = __ballot_sync(0xffffffffu, cand);
-        for (int j = 0; j < 32; ++j) {
-            const double xj = __shfl_sync(0xffffffffu, x, j);
-            if (((m >> j) & 1u) && (kb < 0 || xj > v)) { // a strict > keeps the smallest k
-                v = xj;
-                kb = base + j;
+    __shared__ int kwin;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (wid == 0) {
+        // order keys compare as integers (FP64 compares of one CP after the other took 10 us; the
+        // chain's prices are never NaN nor -0)
+        uint64_t bk = 0;
+        int kb = -1;
+        for (int k = lane; k < g.K; k += 32) // k ascending: a strict > keeps the smallest k
+            if (!occupied[k] && cp_ok[k]) {
+                const uint64_t x = order_key(cp_val[k]);
+                if (kb < 0 || x > bk) {
+                    bk = x;
+                    kb = k;
+                }
+            }
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) {
+            const uint64_t ok = __shfl_xor_sync(0xffffffffu, bk, d);
+            const int o = __shfl_xor_sync(0xffffffffu, kb, d);
+            if (o >= 0 && (kb < 0 || ok > bk || (ok == bk && o < kb))) {
+                bk = ok;
+                kb = o;
             }
         }
+        if (lane == 0) {
+            *best_cp = kb;
+            *best_price = kb >= 0 ? key_value(bk) : -INFINITY;
+            kwin = kb;
+        }
     }
-    if (lane != 0) return;
-    *best_cp = kb;
-    *best_price = kb >= 0 ? v : -INFINITY;
+    __syncthreads();
+    const int kb = kwin;
     if (kb < 0) return;
+    // The backtrack reads one entry of every row's table, each where the one before points: from
+    // global memory 64 accesses one after the other (45 us at 64 rows of 64 columns).
+    // The tables come to shared memory instead, PICK_ROWS rows at a time in 16-byte loads from
+    // the boundary at or before their start, and the walk costs a shared-memory access per row.
+    extern __shared__ __align__(16) int16_t pick_tab[]; // up to 7 entries of the boundary, [PICK_ROWS][NS]
     const int N = g.n_cols;
     const int64_t NS = (int64_t)(N + 1) * (N + 1);
     const int16_t *pt = pred_all + (int64_t)kb * (g.n_rows * NS + 1);
     int cur = pt[g.n_rows * NS];
-    for (int r = g.n_rows - 1; r >= 0; --r) {
-        best_leaves[2 * r] = (int16_t)(cur / (N + 1));
-        best_leaves[2 * r + 1] = (int16_t)(cur % (N + 1));
-        if (r > 0) cur = pt[(int64_t)r * NS + cur];
+    for (int r1 = g.n_rows; r1 > 0; r1 -= PICK_ROWS) {
+        const int r0 = max(r1 - PICK_ROWS, 0);
+        const int n = (int)((r1 - r0) * NS);
+        const int16_t *src = pt + (int64_t)r0 * NS;
+        // (up to 14 bytes past the rows are read too: the table's end and the flags after it)
+        const int mis = (int)((reinterpret_cast<uintptr_t>(src) & 15) / sizeof(int16_t));
+        const uint4 *src4 = reinterpret_cast<const uint4 *>(src - mis);
+        for (int i = threadIdx.x; i < (n + mis + 7) / 8; i += PICK_THREADS) reinterpret_cast<uint4 *>(pick_tab)[i] = src4[i];
+        __syncthreads();
+        if (wid == 0)
+            for (int r = r1 - 1; r >= r0; --r) {
+                if (lane == 0) {
+                    best_leaves[2 * r] = (int16_t)(cur / (N + 1));
+                    best_leaves[2 * r + 1] = (int16_t)(cur % (N + 1));
+                }
+                if (r > 0) cur = pick_tab[mis + (int)((r - r0) * NS) + cur];
+            }
+        __syncthreads();
     }
 }
 
@@ -1019,7 +1091,9 @@ vmat_status pricing_attributes() {
         if (err == cudaSuccess)
             err = cudaFuncSetAttribute(price_cps_interdig_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)interdig_smem(INTERDIG_MAX_COLS));
-
+        if (err == cudaSuccess)
+            err = cudaFuncSetAttribute(price_pick_interdig_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)pick_smem(INTERDIG_MAX_COLS));
     });
     if (err != cudaSuccess)
         return set_error(VMAT_ECUDA, "pricing: cudaFuncSetAttribute failed: %s", cudaGetErrorString(err));
@@ -1111,6 +1185,12 @@ static vmat_status interdig_wave(size_t smem, int *B) {
     return VMAT_OK;
 }
 
+// Blocks of 128 threads of window_prefix_kernel: a warp per 32 rows of a CP.
+static unsigned prefix_grid(const PricingGeom &g) {
+    const int64_t warps = (int64_t)g.K * ((g.n_rows + 31) / 32);
+    return (unsigned)std::max<int64_t>(1, std::min<int64_t>((warps + 3) / 4, 4096));
+}
+
 vmat_status price_apertures_impl(const vmat_mlc *mlc, const float *pi, const uint8_t *occupied, const int16_t *leaves,
                                  int32_t *best_cp, int16_t *best_leaves, double *best_price, void *ws,
                                  cudaStream_t s, const int32_t *skip, bool ws_has_prefix) {
@@ -1126,8 +1206,7 @@ vmat_status price_apertures_impl(const vmat_mlc *mlc, const float *pi, const uin
         VMAT_TRY(pricing_attributes());
         int B = 0;
         VMAT_TRY(interdig_wave(sm, &B));
-        window_prefix_kernel<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>((rows + 127) / 128, 4096)), 128, 0,
-                                 s>>>(g, pi, occupied, leaves, x.Pall, skip);
+        window_prefix_kernel<<<prefix_grid(g), 128, 0, s>>>(g, pi, occupied, leaves, x.Pall, skip);
         VMAT_LAUNCH_CHECK();
         interdig_setup_kernel<<<1, ID_SEL_THREADS, 0, s>>>(g, occupied, x.cp_ok, x.ctl, B, skip);
         VMAT_LAUNCH_CHECK();
@@ -1151,7 +1230,7 @@ vmat_status price_apertures_impl(const vmat_mlc *mlc, const float *pi, const uin
                 g, x.Pall, occupied, leaves, x.cp_val, x.cp_ok, x.pred_all, skip, x.cand2, x.ctl + IDC_N2);
             VMAT_LAUNCH_CHECK();
         }
-        price_pick_interdig_kernel<<<1, 32, 0, s>>>(g, occupied, x.cp_val, x.cp_ok, x.pred_all, best_cp, best_leaves,
+        price_pick_interdig_kernel<<<1, PICK_THREADS, pick_smem(g.n_cols), s>>>(g, occupied, x.cp_val, x.cp_ok, x.pred_all, best_cp, best_leaves,
                                                     best_price, skip);
         VMAT_LAUNCH_CHECK();
         return VMAT_OK;
@@ -1162,8 +1241,7 @@ vmat_status price_apertures_impl(const vmat_mlc *mlc, const float *pi, const uin
     double *Pall = nullptr;
     if (ws_has_prefix) { // after the row bests (pricing_scratch_bytes_prefix)
         Pall = reinterpret_cast<double *>(static_cast<char *>(ws) + row_best_bytes(rows));
-        window_prefix_kernel<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>((rows + 127) / 128, 4096)), 128, 0,
-                               s>>>(g, pi, occupied, leaves, Pall, skip);
+        window_prefix_kernel<<<prefix_grid(g), 128, 0, s>>>(g, pi, occupied, leaves, Pall, skip);
         VMAT_LAUNCH_CHECK();
     }
     price_rows_kernel<<<(unsigned)blocks, PR_WARPS * 32, smem, s>>>(g, pi, occupied, leaves, rb_v, rb_lr, rb_ok, skip,
