@@ -286,7 +286,9 @@ extern "C" vmat_status cg_plan(vmat_ddc hd, const vmat_mlc *mlc, const vmat_voxe
     }
     VMAT_CUDA(cudaMemsetAsync(live_flag, 0, (size_t)n_wtiles, s));
     VMAT_CUDA(cudaMemsetAsync(live.gmask, 0, (size_t)n_wtiles * sizeof(uint32_t), s));
-    VMAT_TRY(inactive_objective(h, vox, F0, s));
+    // (this and the objectives below use the plan's scratch: the stream-ordered pool gives its
+    // memory back whenever the device is synchronised, and mapping it again took 100-200 us each)
+    VMAT_TRY(inactive_objective(h, vox, F0, s, obj_ws));
     VMAT_TRY(ddc_cp_table(h, K, bpc, s)); // CP offsets of CSR(D) rows for the aperture dose
     double F_offset = 0.0;
     VMAT_CUDA(cudaMemcpyAsync(&F_offset, F0, sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -426,7 +428,7 @@ extern "C" vmat_status cg_plan(vmat_ddc hd, const vmat_mlc *mlc, const vmat_voxe
         tm.mark(PH_REFINE);
         // the objective the low-precision master problem reached (its compact dose, plus
         // the constant penalty of the voxels without entries)
-        VMAT_TRY(objective_impl(NA, z_c, h.act_vox, vox, nullptr, nullptr, F_dev + 1, F_offset, s));
+        VMAT_TRY(objective_impl_ws(NA, z_c, h.act_vox, vox, nullptr, nullptr, F_dev + 1, F_offset, obj_ws, s, nullptr));
         for (int t = 0; t < n_placed; ++t) {
             VMAT_TRY(aperture_dose_dev(hf, mlc, cps_dev + t, leaves_seq + (size_t)t * NR * 2,
                                        DA + 32 + (size_t)(t >> 2) * 128 + (t & 3), wstride, nullptr, s));
@@ -451,7 +453,7 @@ extern "C" vmat_status cg_plan(vmat_ddc hd, const vmat_mlc *mlc, const vmat_voxe
     tm.mark(PH_FINAL);
     VMAT_TRY(aperture_fluence(mlc, n_apertures, cps_dev, leaves_seq, y, x, s));
     VMAT_TRY(dose_forward_impl(refine ? hf : h, x, dose, false, s));
-    VMAT_TRY(objective_impl(V, dose, nullptr, vox, nullptr, nullptr, F_dev, 0.0, s));
+    VMAT_TRY(objective_impl_ws(V, dose, nullptr, vox, nullptr, nullptr, F_dev, 0.0, obj_ws, s, nullptr));
     tm.end();
     VMAT_CUDA(cudaEventRecord(t1, s));
     VMAT_CUDA(cudaMemcpyAsync(hctl, ctl, CTL_N * sizeof(int32_t), cudaMemcpyDeviceToHost, s));

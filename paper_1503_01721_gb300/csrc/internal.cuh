@@ -422,7 +422,8 @@ vmat_status objective_impl_ws(int32_t n, const float *z, const int32_t *idx, con
                               const int32_t *skip, const int32_t *gpos = nullptr);
 size_t objective_scratch_bytes(int n_sm);
 // F0 = the penalty at zero dose of the voxels without DDC entries (their dose is always 0).
-vmat_status inactive_objective(const Ddc &h, const vmat_voxels *vox, double *F0, cudaStream_t s);
+// ws: scratch of objective_scratch_bytes, or null (stream-ordered scratch of its own).
+vmat_status inactive_objective(const Ddc &h, const vmat_voxels *vox, double *F0, cudaStream_t s, void *ws = nullptr);
 
 // compact: write row r of CSR(D) (wstride == 0: at da[r]; else at da[(r / 32) * wstride + (r % 32) * 4],
 // the master problem's warp-tile layout with da pointing at the column's first slot);

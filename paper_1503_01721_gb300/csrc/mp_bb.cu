@@ -2126,6 +2126,40 @@ vmat_status mp_bb_enqueue_batched(const void *args, const int64_t *weight, unsig
     return VMAT_OK;
 }
 
+// Scratch of mp_bb_impl that a thread keeps between calls: the call returns only after its
+// stream has been synchronised, so the next call of the thread may use it on any stream.
+// At most MP_KEEP_BYTES; freed when the thread ends, or when a larger one or another device is
+// needed.  (From the stream-ordered pool, which gives its memory back at each synchronisation,
+// the 70 MB of a 422K-voxel, 40-aperture problem were mapped anew in every call.)
+constexpr size_t MP_KEEP_BYTES = (size_t)128 << 20;
+struct MpKeep {
+    void *p = nullptr;
+    size_t bytes = 0;
+    int dev = -1;
+    void drop() {
+        if (p) cudaFree(p);
+        p = nullptr;
+        bytes = 0;
+        dev = -1;
+    }
+    ~MpKeep() { drop(); }
+};
+static void *mp_keep(size_t bytes, int dev) {
+    static thread_local MpKeep k;
+    if (bytes > MP_KEEP_BYTES) return nullptr;
+    if (k.dev != dev || k.bytes < bytes) {
+        k.drop();
+        if (cudaMalloc(&k.p, bytes) != cudaSuccess) {
+            cudaGetLastError();
+            k.p = nullptr;
+            return nullptr;
+        }
+        k.bytes = bytes;
+        k.dev = dev;
+    }
+    return k.p;
+}
+
 vmat_status mp_bb_impl(const float *DA, int32_t V, int32_t n_ap, int64_t ld, const uint8_t *struct_id,
                        int64_t wstride, const vmat_voxels *vox, const float *lo, const float *hi, float *y,
                        float *z, const vmat_bb_opts *opts_in, double F_offset, vmat_bb_report *rep, cudaStream_t s) {
@@ -2137,31 +2171,37 @@ vmat_status mp_bb_impl(const float *DA, int32_t V, int32_t n_ap, int64_t ld, con
     if (ldg_smem(n_ap) > MP_SMEM_LIMIT) return set_error(VMAT_EUNSUPPORTED, "mp_bb_solve: too many apertures (%d)", n_ap);
     const int64_t n_wtiles = ((int64_t)V + MP_WT - 1) / MP_WT;
 
-    // a column-major input is copied once into the warp-tile layout (with the labels)
-    Scratch conv;
-    if (wstride == 0) {
-        wstride = mp_wtile_stride(n_ap);
-        VMAT_TRY(conv.alloc((size_t)n_wtiles * wstride * sizeof(float), s));
-        const int64_t total = n_wtiles * wstride;
-        const int g = (int)std::max<int64_t>(1, std::min<int64_t>((total + 255) / 256, (int64_t)ctx->n_sm * 16));
-        to_warp_tiles<<<g, 256, 0, s>>>(DA, ld, V, n_ap, struct_id, wstride, n_wtiles, static_cast<float *>(conv.ptr));
-        VMAT_LAUNCH_CHECK();
-        DA = static_cast<const float *>(conv.ptr);
-    }
     MPLaunch L;
     VMAT_TRY(mp_configure(V, n_ap, ctx, &L));
     const int p_max = std::max(mp_p_max(ctx), std::max(L.P, L.Pc));
-    Scratch ws;
-    VMAT_TRY(ws.alloc(mp_ws_bytes(n_ap, p_max), s));
+    const size_t conv_bytes =
+        wstride == 0 ? (((size_t)n_wtiles * mp_wtile_stride(n_ap) * sizeof(float) + 255) & ~(size_t)255) : 0;
+    const size_t bytes = conv_bytes + mp_ws_bytes(n_ap, p_max);
+    Scratch own; // when the thread's kept scratch does not hold it
+    void *mem = mp_keep(bytes, ctx->device);
+    if (!mem) {
+        VMAT_TRY(own.alloc(bytes, s));
+        mem = own.ptr;
+    }
+    void *const ws = static_cast<char *>(mem) + conv_bytes;
+    // a column-major input is copied once into the warp-tile layout (with the labels)
+    if (wstride == 0) {
+        wstride = mp_wtile_stride(n_ap);
+        const int64_t total = n_wtiles * wstride;
+        const int g = (int)std::max<int64_t>(1, std::min<int64_t>((total + 255) / 256, (int64_t)ctx->n_sm * 16));
+        to_warp_tiles<<<g, 256, 0, s>>>(DA, ld, V, n_ap, struct_id, wstride, n_wtiles, static_cast<float *>(mem));
+        VMAT_LAUNCH_CHECK();
+        DA = static_cast<const float *>(mem);
+    }
     MPArgs a;
-    mp_fill_args(a, ws.ptr, n_ap, p_max, DA, wstride, V, n_ap, struct_id, vox, lo, hi, y, z, opts, F_offset, L, ctx);
+    mp_fill_args(a, ws, n_ap, p_max, DA, wstride, V, n_ap, struct_id, vox, lo, hi, y, z, opts, F_offset, L, ctx);
     const size_t smem_cauchy = (size_t)((n_ap + 3) & ~3) * 4 + 3 * 256 * 4;
 
     static thread_local BBState *host_st = nullptr;
     if (!host_st) VMAT_CUDA(cudaMallocHost(&host_st, sizeof(BBState)));
 
     if (L.persistent) {
-        VMAT_CUDA(cudaMemsetAsync(ws.ptr, 0, mp_zero_bytes(n_ap, p_max), s));
+        VMAT_CUDA(cudaMemsetAsync(ws, 0, mp_zero_bytes(n_ap, p_max), s));
         VMAT_TRY(mp_launch_persistent(a, L, s));
         VMAT_CUDA(cudaMemcpyAsync(host_st, a.st, sizeof(BBState), cudaMemcpyDeviceToHost, s));
         VMAT_CUDA(cudaStreamSynchronize(s));

@@ -170,16 +170,18 @@ vmat_status objective_impl(int32_t n, const float *z, const int32_t *idx, const 
     return objective_impl_ws(n, z, idx, vox, g, g_scatter, F, F_offset, ws.ptr, s, nullptr);
 }
 
-vmat_status inactive_objective(const Ddc &h, const vmat_voxels *vox, double *F0, cudaStream_t s) {
+vmat_status inactive_objective(const Ddc &h, const vmat_voxels *vox, double *F0, cudaStream_t s, void *ws_in) {
     DeviceCtx *ctx;
     VMAT_TRY(device_ctx(&ctx));
     const int grid = obj_grid(h.V, ctx->n_sm);
     Scratch ws;
-    VMAT_TRY(ws.alloc((size_t)grid * sizeof(double), s));
+    if (!ws_in) VMAT_TRY(ws.alloc((size_t)grid * sizeof(double), s));
+    // the partials' place in objective_scratch_bytes (its first 64 bytes are the counter's)
+    double *partial = ws_in ? reinterpret_cast<double *>(static_cast<char *>(ws_in) + 64) : (double *)ws.ptr;
     inactive_objective_kernel<<<grid, OBJ_THREADS, 0, s>>>(h.V, h.vox2act, vox->struct_id, vox->T, vox->w_over,
-                                                           vox->w_under, (double *)ws.ptr);
+                                                           vox->w_under, partial);
     VMAT_LAUNCH_CHECK();
-    sum_partials<<<1, OBJ_THREADS, 0, s>>>((double *)ws.ptr, grid, F0);
+    sum_partials<<<1, OBJ_THREADS, 0, s>>>(partial, grid, F0);
     VMAT_LAUNCH_CHECK();
     return VMAT_OK;
 }
