@@ -631,11 +631,32 @@ __device__ __forceinline__ float warp_row_sum_x(const int64_t *__restrict__ rowp
 // list items in runs of WIN_RUN consecutive items, run warp0, warp0 + stride, ...; the
 // items of a run are consecutive rows of one window segment or of the next ones, so
 // the segment is searched once per run and then followed item by item.
+// With a CP mask over at most ACT_MAX CPs (act, from active_cps): the rows of the active CPs
+// only, numbered without the others, so that every warp gets as many.  (Rows warp0,
+// warp0 + stride, ... with the masked ones skipped left the warp whose rows all fell into active
+// CPs to finish alone.)
 constexpr int WIN_RUN = 4;
-template <typename F> __device__ __forceinline__ void for_rows(const RowParams &p, int64_t warp0, F &&f) {
-    if (!p.mask.woff) {
-        for (int64_t r = warp0; r < p.n_rows; r += p.stride)
-            if (row_needed(p.mask, r)) f(r);
+constexpr int ACT_MAX = 1024;
+struct ActiveCps {
+    int n; // active CPs, or -1: no list
+    uint16_t cp[ACT_MAX];
+    int count[ACT_MAX / 32];
+};
+template <typename F>
+__device__ __forceinline__ void for_rows(const RowParams &p, const ActiveCps &act, int64_t warp0, F &&f) {
+    if (!p.mask.woff) { // one call of f for both numberings: a second one would cost registers
+        const bool list = act.n >= 0;
+        const int64_t n = list ? (int64_t)act.n * p.mask.bpc : (int64_t)p.n_rows;
+        for (int64_t i = warp0; i < n; i += p.stride) {
+            int64_t r = i;
+            if (list) {
+                const int32_t q = (int32_t)i / p.mask.bpc;
+                r = (int64_t)act.cp[q] * p.mask.bpc + ((int32_t)i - q * p.mask.bpc);
+            } else if (!row_needed(p.mask, r)) {
+                continue;
+            }
+            f(r);
+        }
         return;
     }
     const int64_t n_items = (int64_t)__ldg(p.mask.woff + p.mask.nseg);
@@ -660,14 +681,48 @@ template <typename F> __device__ __forceinline__ void for_rows(const RowParams &
     }
 }
 
+// The active CPs in ascending order (the whole block, once per launch: a flag per thread and
+// load, ballots, the warps' counts in order).
+template <int THREADS> __device__ __forceinline__ void active_cps(const RowParams &p, ActiveCps &act) {
+    const int lane = threadIdx.x & 31;
+    const int K = p.mask.cp_active && !p.mask.win ? p.n_rows / max(p.mask.bpc, 1) : ACT_MAX + 1;
+    if (K > ACT_MAX) { // block-uniform
+        if (threadIdx.x == 0) act.n = -1;
+        __syncthreads();
+        return;
+    }
+    for (int k0 = 0; k0 < ACT_MAX; k0 += THREADS) {
+        const int k = k0 + threadIdx.x;
+        const unsigned m = __ballot_sync(0xffffffffu, k < K && p.mask.cp_active[min(k, K - 1)]);
+        if (lane == 0) act.count[k >> 5] = __popc(m);
+    }
+    __syncthreads();
+    for (int k0 = 0; k0 < K; k0 += THREADS) {
+        const int k = k0 + threadIdx.x;
+        const bool on = k < K && p.mask.cp_active[min(k, K - 1)];
+        const unsigned m = __ballot_sync(0xffffffffu, on);
+        int at = 0;
+        for (int w = 0; w < (k >> 5); ++w) at += act.count[w];
+        if (on) act.cp[at + __popc(m & ((1u << lane) - 1u))] = (uint16_t)k;
+    }
+    if (threadIdx.x == 0) {
+        int n = 0;
+        for (int w = 0; w < (K + 31) / 32; ++w) n += act.count[w];
+        act.n = n;
+    }
+    __syncthreads();
+}
+
 template <int THREADS, int UNROLL, typename VT>
 __global__ void __launch_bounds__(THREADS) spmv_warp_row_z_kernel(RowParams p) {
     if (p.skip && *p.skip) return;
+    __shared__ ActiveCps act;
+    active_cps<THREADS>(p, act);
     const int lane = threadIdx.x & 31;
     const int64_t warp0 = ((int64_t)blockIdx.x * THREADS + threadIdx.x) >> 5;
-    if (warp0 >= p.stride) return; // warp-uniform
+    if (warp0 >= p.stride) return; // warp-uniform, after the block's barriers
     const uint64_t pol = l2_evict_first_policy();
-    for_rows(p, warp0, [&](int64_t r) {
+    for_rows(p, act, warp0, [&](int64_t r) {
         float sum = warp_row_sum_z<UNROLL, VT>(p.rowptr, p.cptr, p.cbase, p.col16, p.val, p.x, r, lane, pol);
         if (lane == 0) {
             if (p.row_scale) sum *= p.row_scale[r];
@@ -679,11 +734,13 @@ __global__ void __launch_bounds__(THREADS) spmv_warp_row_z_kernel(RowParams p) {
 template <int THREADS, int CTAS, typename VT>
 __global__ void __launch_bounds__(THREADS, CTAS) spmv_warp_row_x_kernel(RowParams p) {
     if (p.skip && *p.skip) return;
+    __shared__ ActiveCps act;
+    active_cps<THREADS>(p, act);
     const int lane = threadIdx.x & 31;
     const int64_t warp0 = ((int64_t)blockIdx.x * THREADS + threadIdx.x) >> 5;
-    if (warp0 >= p.stride) return; // warp-uniform
+    if (warp0 >= p.stride) return; // warp-uniform, after the block's barriers
     const uint64_t pol = l2_evict_first_policy();
-    for_rows(p, warp0, [&](int64_t r) {
+    for_rows(p, act, warp0, [&](int64_t r) {
         float sum = warp_row_sum_x<VT>(p.rowptr, p.col, p.strm, p.sptr, p.x, r, lane, pol);
         if (lane == 0) {
             if (p.row_scale) sum *= p.row_scale[r];
@@ -695,11 +752,13 @@ __global__ void __launch_bounds__(THREADS, CTAS) spmv_warp_row_x_kernel(RowParam
 template <int THREADS, int UNROLL, typename VT>
 __global__ void __launch_bounds__(THREADS) spmv_warp_row_c_kernel(RowParams p) {
     if (p.skip && *p.skip) return;
+    __shared__ ActiveCps act;
+    active_cps<THREADS>(p, act);
     const int lane = threadIdx.x & 31;
     const int64_t warp0 = ((int64_t)blockIdx.x * THREADS + threadIdx.x) >> 5;
-    if (warp0 >= p.stride) return; // warp-uniform
+    if (warp0 >= p.stride) return; // warp-uniform, after the block's barriers
     const uint64_t pol = l2_evict_first_policy();
-    for_rows(p, warp0, [&](int64_t r) {
+    for_rows(p, act, warp0, [&](int64_t r) {
         float sum = warp_row_sum_c<UNROLL, VT>(p.rowptr, p.col, p.val, p.x, r, lane, pol);
         if (lane == 0) {
             if (p.row_scale) sum *= p.row_scale[r];
@@ -711,11 +770,13 @@ __global__ void __launch_bounds__(THREADS) spmv_warp_row_c_kernel(RowParams p) {
 template <int THREADS, int UNROLL, typename VT>
 __global__ void __launch_bounds__(THREADS) spmv_warp_row_kernel(RowParams p) {
     if (p.skip && *p.skip) return;
+    __shared__ ActiveCps act;
+    active_cps<THREADS>(p, act);
     const int lane = threadIdx.x & 31;
     const int64_t warp0 = ((int64_t)blockIdx.x * THREADS + threadIdx.x) >> 5;
-    if (warp0 >= p.stride) return; // warp-uniform
+    if (warp0 >= p.stride) return; // warp-uniform, after the block's barriers
     const uint64_t pol = l2_evict_first_policy();
-    for_rows(p, warp0, [&](int64_t r) {
+    for_rows(p, act, warp0, [&](int64_t r) {
         float sum = warp_row_sum<UNROLL, VT>(p.rowptr, p.col, p.val, p.x, r, lane, pol);
         if (lane == 0) {
             if (p.row_scale) sum *= p.row_scale[r];

@@ -60,3 +60,24 @@ def test_same_bits_as_the_16_bit_index_and_zero_padding_is_not_read(dtype):
         a = _products(make_ddc(c, dtype, z, brick=True), c.V, c.J, g, x)
         b = _products(make_ddc(c, dtype, twin, brick=True), c.V, c.J, g, x)
         assert all(np.array_equal(u.view(np.uint32), v.view(np.uint32)) for u, v in zip(a, b))
+
+
+@pytest.mark.parametrize("K,bpc,cfg", [(1, 16, 9), (31, 8, 4), (33, 5, 9), (256, 3, 11), (257, 4, 10), (1024, 1, 9),
+                                       (1025, 2, 5)])  # at most 1024 CPs: a list of the active ones
+def test_rows_of_the_active_cps(K, bpc, cfg):
+    """Every row of the active CPs and no other is written, with the full pass's bits."""
+    require_cuda()
+    from paper_1503_01721_gb300 import api
+    rng = np.random.default_rng(K)
+    V, J = 500, K * bpc
+    blt = np.repeat(np.arange(J, dtype=np.int32), 6)
+    vox = np.concatenate([np.sort(rng.choice(V, 6, replace=False)) for _ in range(J)]).astype(np.int32)
+    ddc = make_ddc((vox, blt, rng.uniform(0.1, 1, len(vox)).astype(np.float32)), "f32", cfg, V, J)
+    g = dev(synth.random_vector(V, 3), torch.float32)
+    full = torch.empty(J, device="cuda")
+    api.beamlet_price(ddc.h, g, full)
+    for active in (rng.random(K) < 0.5, np.zeros(K, bool), np.ones(K, bool)):
+        pi = torch.full((J,), 7.0, device="cuda")
+        api.beamlet_price(ddc.h, g, pi, dev(active.astype(np.uint8), torch.uint8), bpc)
+        want = np.where(np.repeat(active, bpc), host(full), np.float32(7.0))
+        assert np.array_equal(host(pi).view(np.uint32), want.view(np.uint32))
