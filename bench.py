@@ -49,17 +49,18 @@ WORKLOAD_DESC = DESCS[WORKLOAD]
 SPMV_KERNELS = {0: "spmv_tile_kernel<256,16,2>", 1: "spmv_tile_kernel<256,8,3>", 2: "spmv_tile_kernel<512,8,2>",
                 3: "spmv_tile_kernel<128,16,3>", 4: "spmv_warp_row_kernel<256,2>", 5: "spmv_warp_row_kernel<256,1>",
                 6: "spmv_warp_row_kernel<512,4>", 7: "spmv_warp_row_kernel<256,4>", 8: "spmv_warp_row_kernel<256,8>",
-                9: "spmv_warp_row_c_kernel<256,4>", 10: "spmv_warp_row_c_kernel<256,8>",
-                11: "spmv_warp_row_c_kernel<512,4>", 12: "spmv_warp_row_z_kernel<256,4>",
+                # 9-11 read the packed stream of the matrix (spmv_warp_row_c_kernel where there is none)
+                9: "spmv_warp_row_x_kernel<256,8>", 10: "spmv_warp_row_x_kernel<256,6>",
+                11: "spmv_warp_row_x_kernel<512,4>", 12: "spmv_warp_row_z_kernel<256,4>",
                 13: "spmv_warp_row_z_kernel<256,8>", 14: "spmv_warp_row_z_kernel<512,4>"}
 # configurations that read the 16-bit column index (built with index16)
 INDEX16_CFGS = (12, 13, 14)
 # DRAM traffic over algorithmic bytes of the plan's windowed D^T g launches, per (value type,
 # configuration, CSR(D^T) column order): dram__bytes_read.sum + dram__bytes_write.sum over the 30
 # windowed launches of the 45-CP plan (the same kernels on a quarter of the CPs), over their algorithmic
-# bytes, from one ncu capture each; a configuration without such a capture reports null.
-WINDOWED_TRAFFIC_RATIO = {("f32", 5, "voxel"): 0.9988, ("f32", 9, "voxel"): 1.0010, ("f32", 11, "voxel"): 1.0009,
-                          ("f32", 9, "brick"): 1.0039, ("f32", 11, "brick"): 1.0038}
+# bytes, from one ncu capture each; a configuration without such a capture reports null
+# (configurations 9-11 since they read the packed stream).
+WINDOWED_TRAFFIC_RATIO = {("f32", 5, "voxel"): 0.9988}
 # The paper's own plan times (Table 2 and Table 3): other hardware, patient data and aperture
 # counts, so context for the line, not a baseline of its metric.
 PAPER_CONTEXT = {

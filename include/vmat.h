@@ -98,7 +98,12 @@ typedef struct {
     int32_t build_Dt;   /* nonzero: build CSR(D^T), beamlet rows (beamlet_price) */
     int32_t tile_cfg;   /* SpMV configuration index of CSR(D) (and of CSR(D^T) when tile_cfg_Dt < 0),
                            -1 = library default */
-    int32_t autotune;   /* nonzero: time every tile configuration and keep the fastest */
+    int32_t autotune;   /* nonzero: time every tile configuration and keep the fastest.  Such a build,
+                           and one with a consecutive-lane configuration (9-11), also holds each CSR as
+                           a packed stream that those configurations read (records of 128 entries with
+                           16-bit column offsets: s_val + 2.1 bytes per entry, rows padded to whole
+                           records; same sums, same bits), where memory allows and the columns of
+                           nearly every 32 entries span fewer than 65,536 */
     int32_t keep_coo;   /* nonzero: keep the COO copy after the build */
     int32_t index16;    /* nonzero: also store 16-bit column indices (rows cut into 128-entry
                            chunks, each with a 32-bit base column) for every CSR whose chunks all
@@ -335,7 +340,8 @@ vmat_status aperture_grad(const vmat_mlc *mlc, int32_t n_ap, const int32_t *cps,
  * solution out.  z: device float [V], receives DA y.  opts NULL = defaults
  * (500, 1e-6, 1e-9, 1e-12, 1e12).  rep: HOST struct or NULL.
  * The step lengths, objective and stopping tests use FP64; the products FP32.
- * Synchronises. */
+ * Synchronises.  Scratch of up to 128 MB stays with the calling thread for its next
+ * call (freed when the thread ends); more comes from the stream-ordered pool. */
 vmat_status mp_bb_solve(const float *DA, int32_t V, int32_t n_ap, int64_t ld, const vmat_voxels *vox,
                         const float *lo, const float *hi, float *y, float *z, const vmat_bb_opts *opts,
                         vmat_bb_report *rep, void *stream);

@@ -273,7 +273,9 @@ vmat_status dose_forward_impl(const Ddc &h, const float *x, float *d, bool compa
 // `nnz` nonzeros and `chunks` 16-bit-index chunks, in the format configuration
 // cfg reads: each value (vb bytes) and column index (4, or 2 plus a 4-byte base
 // per chunk and an 8-byte chunk pointer per row) once, an 8-byte row pointer
-// per row.  Dense inputs, outputs and scales are the caller's.
+// per row.  Dense inputs, outputs and scales are the caller's.  Where configurations 9-11 read
+// the packed stream these stay the CSR's bytes (the metric's definition); the stream moves
+// about 0.83 (FP32), 0.78 (BF16) and 0.72 (FP8) of them at 1,300 entries per row.
 inline double csr_pass_bytes(int cfg, int vb, double nnz, double rows, double chunks) {
     if (spmv_config_index16(cfg)) return nnz * (vb + 2) + 4.0 * chunks + 16.0 * rows;
     return nnz * (vb + 4) + 8.0 * rows;
