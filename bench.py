@@ -59,8 +59,8 @@ INDEX16_CFGS = (12, 13, 14)
 # configuration, CSR(D^T) column order): dram__bytes_read.sum + dram__bytes_write.sum over the 30
 # windowed launches of the 45-CP plan (the same kernels on a quarter of the CPs), over their algorithmic
 # bytes, from one ncu capture each; a configuration without such a capture reports null
-# (configurations 9-11 since they read the packed stream).
-WINDOWED_TRAFFIC_RATIO = {("f32", 5, "voxel"): 0.9988}
+# (9 and 10 since they read the packed stream, which moves less than the CSR's bytes).
+WINDOWED_TRAFFIC_RATIO = {("f32", 5, "voxel"): 0.9988, ("f32", 11, "brick"): 0.8407}
 # The paper's own plan times (Table 2 and Table 3): other hardware, patient data and aperture
 # counts, so context for the line, not a baseline of its metric.
 PAPER_CONTEXT = {
