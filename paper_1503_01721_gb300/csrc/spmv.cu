@@ -1268,6 +1268,14 @@ vmat_status spmv_autotune(Ddc &h, cudaStream_t s) {
         cudaFree(x);
         cudaFree(y);
         VMAT_TRY(spmv_prepare_tiles(*m, best, s));
+        // CSR(D) is read in this configuration only; CSR(D^T)'s windowed passes and batches choose their own
+        if (!isDt && m->strm && !spmv_config_stream(best)) {
+            VMAT_CUDA(cudaStreamSynchronize(s));
+            cudaFree(m->strm);
+            cudaFree(m->sptr);
+            m->strm = nullptr;
+            m->sptr = nullptr;
+        }
     }
     VMAT_CUDA(cudaStreamSynchronize(s));
     h.tuned = true;
