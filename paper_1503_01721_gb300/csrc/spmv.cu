@@ -20,6 +20,7 @@
 //      a second small kernel adds carries to their rows in tile order.
 // All orders of addition are fixed, so results are bitwise reproducible.
 #include <algorithm>
+#include <mutex>
 
 #include "internal.cuh"
 
@@ -392,6 +393,7 @@ struct RowParams {
     RowMask mask; // the rows to compute
     int32_t n_rows;
     int64_t stride; // rows between a warp's consecutive rows (<= the launch's warps; warps past it idle)
+    uint32_t step_cps, step_rows; // ROWS_CPS: the stride as whole CPs of mask.bpc rows and the rest
     const int32_t *skip; // when non-null and set, the kernel does nothing
     const unsigned char *strm; // packed stream (spmv_warp_row_x_kernel)
     const int32_t *sptr;
@@ -523,12 +525,18 @@ __device__ __forceinline__ float warp_row_sum_z(const int64_t *__restrict__ rowp
 // 1,024, 768 or 640 bytes and eight.
 //
 // What bounds it: the gathers of x in L1, about two cycles per 128-byte line touched (3.5 lines per
-// 32 entries of a beamlet row in brick order): the times hardly follow the bytes.  So many
-// warps are kept resident (32 registers, 64 warps per SM).  484M nonzeros (128 x 128 x 96
-// voxels, 90 CPs, brick order), the CSR's fastest configuration -> this one: D^T g FP32 0.696 ->
-// 0.620 ms, BF16 0.615 -> 0.520, FP8 0.534 -> 0.491; D x 0.728 -> 0.703, 0.689 -> 0.663, 0.695
-// -> 0.625.  Slower: the next record in flight in registers (48 registers: 0.693 ms FP32), two
-// records at once, and prefetching the next records into L2 (0.678 ms).
+// 32 entries of a beamlet row in brick order), and how many loads are in flight.  So 64 warps are
+// kept resident per SM (32 registers), nothing is spilled, and in FP32 and BF16 a record's bases and
+// offsets are loaded while the gathers of the record before it are under way.  (In FP8 that
+// order came out slower, D^T g 1.00 ms instead of 0.72: there a record is loaded when it is used.)
+// 968M nonzeros (128 x 128 x 96 voxels, 180 CPs, brick order), best of configurations 9-11 from the
+// CSR -> from the stream with the row numberings in one kernel (27 words spilled) -> now, in ms:
+//   D^T g, every row:        FP32 1.28 -> 1.04 -> 0.97, BF16 1.22 -> 0.82 -> 0.72, FP8 1.06 -> 0.77 -> 0.72
+//   D^T g, a third occupied: FP32 0.84 -> 0.68 -> 0.63, BF16 0.82 -> 0.54 -> 0.47, FP8 0.71 -> 0.51 -> 0.47
+//   D^T g, in windows:       FP32 0.53 -> 0.47 -> 0.42, BF16 0.48 -> 0.36 -> 0.33, FP8 0.45 -> 0.34 -> 0.32
+//   D x:                     FP32 1.41 -> 1.45 -> 1.30, BF16 1.37 -> 1.36 -> 1.22, FP8 1.36 -> 1.33 -> 1.26
+// Slower: a record's loads issued together and awaited (FP32 D^T g 0.99, BF16 0.94), two records at
+// a time (1.02, 0.82, with spills), prefetching the next records into L2.
 // (The values stay as loaded until their products: a conversion would wait for the load.)
 template <typename VT> struct RawVals;
 template <> struct RawVals<float> {
@@ -575,30 +583,40 @@ template <typename VT> struct StreamRec {
     RawVals<VT> v;
     uint2 o;
     int4 b;
-    __device__ __forceinline__ void load(const unsigned char *q, int lane, uint64_t pol) {
+    __device__ __forceinline__ void load_index(const unsigned char *q, int lane, uint64_t pol) {
         b = ldg_stream_i4(q, pol);
         o = ldg_stream_u2(q + 16 + lane * 8, pol);
+    }
+    __device__ __forceinline__ void load_values(const unsigned char *q, int lane, uint64_t pol) {
         v.load(q + 16 + STRM_ENTRIES * 2, lane, pol);
     }
 };
-// acc[u] += value * x over one record; left: the row's entries from the record on (> 0), col: their columns.
-template <typename VT>
-__device__ __forceinline__ void record_products(const StreamRec<VT> &q, const int32_t *__restrict__ col, int left,
+// acc[u] += value * x over one record; left: the row's entries from the record on (FULL: at least
+// STRM_ENTRIES of them), row_end: the row's end in col.
+template <bool FULL, typename VT>
+__device__ __forceinline__ void record_products(const StreamRec<VT> &q, const int32_t *__restrict__ col,
+                                                const int64_t *__restrict__ row_end, int left,
                                                 const float *__restrict__ x, int lane, float acc[4]) {
     const int32_t bs[4] = {q.b.x, q.b.y, q.b.z, q.b.w};
     int32_t j[4] = {bs[0] + (int32_t)(q.o.x & 0xffffu), bs[1] + (int32_t)(q.o.x >> 16),
                     bs[2] + (int32_t)(q.o.y & 0xffffu), bs[3] + (int32_t)(q.o.y >> 16)};
     if ((bs[0] | bs[1] | bs[2] | bs[3]) < 0) { // a chunk that spans 65,536 columns or more
+        // (its place in col is found here, from the row's end: kept along, it would cost two registers)
+        const int32_t *c = col + (__ldg(row_end) - left) + lane;
 #pragma unroll
         for (int u = 0; u < 4; ++u)
-            if (bs[u] < 0 && 32 * u + lane < left) j[u] = __ldg(col + 32 * u + lane);
+            if (bs[u] < 0 && (FULL || 32 * u + lane < left)) j[u] = __ldg(c + 32 * u);
     }
     float v[4];
-    q.v.get(v);
-    if (left >= STRM_ENTRIES) {
+    if (FULL) {
+        float xv[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) acc[u] = fmaf(v[u], __ldg(x + j[u]), acc[u]);
+        for (int u = 0; u < 4; ++u) xv[u] = __ldg(x + j[u]);
+        q.v.get(v);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc[u] = fmaf(v[u], xv[u], acc[u]);
     } else {
+        q.v.get(v);
 #pragma unroll
         for (int u = 0; u < 4; ++u)
             if (32 * u + lane < left) acc[u] = fmaf(v[u], __ldg(x + j[u]), acc[u]);
@@ -610,15 +628,43 @@ __device__ __forceinline__ float warp_row_sum_x(const int64_t *__restrict__ rowp
                                                 const int32_t *__restrict__ sptr, const float *__restrict__ x,
                                                 int64_t r, int lane, uint64_t pol) {
     constexpr int REC = strm_record_bytes((int)sizeof(VT));
-    const int64_t s = __ldg(rowptr + r);
-    int n = (int)(__ldg(rowptr + r + 1) - s);
-    const unsigned char *rec = strm + (int64_t)__ldg(sptr + r) * REC;
-    const int32_t *c = col + s;
+    const int64_t *row_end = rowptr + r + 1;
+    int n = (int)(__ldg(row_end) - __ldg(rowptr + r));
     float acc[4] = {0.f, 0.f, 0.f, 0.f};
-    for (; n > 0; n -= STRM_ENTRIES, rec += REC, c += STRM_ENTRIES) {
+    if constexpr (sizeof(VT) > 1) { // the next record's bases and offsets in flight with this one's gathers
+        uint32_t i = (uint32_t)__ldg(sptr + r);
         StreamRec<VT> q;
-        q.load(rec, lane, pol);
-        record_products<VT>(q, c, n, x, lane, acc);
+        q.b = make_int4(0, 0, 0, 0);
+        q.o = make_uint2(0, 0);
+        if (n > 0) q.load_index(strm + (size_t)i * REC, lane, pol);
+#pragma unroll 1
+        for (; n > STRM_ENTRIES; n -= STRM_ENTRIES) {
+            StreamRec<VT> now;
+            now.b = q.b;
+            now.o = q.o;
+            now.load_values(strm + (size_t)i * REC, lane, pol);
+            ++i;
+            q.load_index(strm + (size_t)i * REC, lane, pol);
+            record_products<true, VT>(now, col, row_end, n, x, lane, acc);
+        }
+        if (n > 0) { // the row's last record, padded
+            q.load_values(strm + (size_t)i * REC, lane, pol);
+            record_products<false, VT>(q, col, row_end, n, x, lane, acc);
+        }
+    } else {
+        const unsigned char *rec = strm + (int64_t)__ldg(sptr + r) * REC;
+        StreamRec<VT> q;
+#pragma unroll 1
+        for (; n >= STRM_ENTRIES; n -= STRM_ENTRIES, rec += REC) {
+            q.load_index(rec, lane, pol);
+            q.load_values(rec, lane, pol);
+            record_products<true, VT>(q, col, row_end, n, x, lane, acc);
+        }
+        if (n > 0) { // the row's last record, padded
+            q.load_index(rec, lane, pol);
+            q.load_values(rec, lane, pol);
+            record_products<false, VT>(q, col, row_end, n, x, lane, acc);
+        }
     }
     float sum = (acc[0] + acc[1]) + (acc[2] + acc[3]);
 #pragma unroll
@@ -626,71 +672,34 @@ __device__ __forceinline__ float warp_row_sum_x(const int64_t *__restrict__ rowp
     return sum;
 }
 
-// The rows of a warp-row launch, passed to f in order.  Without a list: rows
-// warp0, warp0 + stride, ... that the mask keeps.  With the window list (mask.woff):
-// list items in runs of WIN_RUN consecutive items, run warp0, warp0 + stride, ...; the
-// items of a run are consecutive rows of one window segment or of the next ones, so
-// the segment is searched once per run and then followed item by item.
-// With a CP mask over at most ACT_MAX CPs (act, from active_cps): the rows of the active CPs
-// only, numbered without the others, so that every warp gets as many.  (Rows warp0,
-// warp0 + stride, ... with the masked ones skipped left the warp whose rows all fell into active
-// CPs to finish alone.)
+// The rows of a warp-row launch, in one of three numberings.  The kernels take the numbering
+// as a template argument, chosen by the launch (numbering_of), so that each holds the registers
+// and the shared memory of its own only.
+//   ROWS_ALL: rows warp0, warp0 + stride, ... that the mask keeps.
+//   ROWS_WINDOWS (mask.woff): list items in runs of WIN_RUN consecutive items, run warp0, warp0 +
+//     stride, ...; the items of a run are consecutive rows of one window segment or of the next
+//     ones, so the segment is searched once per run and then followed item by item.
+//   ROWS_CPS (a CP mask over at most ACT_MAX CPs): the rows of the active CPs only, numbered
+//     without the others, so that every warp gets as many.  (Rows warp0, warp0 + stride, ... with the
+//     masked ones skipped left the warp whose rows all fell into active CPs to finish alone.)
+enum Numbering { ROWS_ALL = 0, ROWS_WINDOWS = 1, ROWS_CPS = 2, N_NUMBERINGS = 3 };
 constexpr int WIN_RUN = 4;
 constexpr int ACT_MAX = 1024;
+static Numbering numbering_of(const RowMask &m, int32_t n_rows) {
+    if (m.woff) return ROWS_WINDOWS;
+    return m.cp_active && !m.win && n_rows / std::max(m.bpc, 1) <= ACT_MAX ? ROWS_CPS : ROWS_ALL;
+}
 struct ActiveCps {
-    int n; // active CPs, or -1: no list
+    int n; // active CPs
     uint16_t cp[ACT_MAX];
     int count[ACT_MAX / 32];
 };
-template <typename F>
-__device__ __forceinline__ void for_rows(const RowParams &p, const ActiveCps &act, int64_t warp0, F &&f) {
-    if (!p.mask.woff) { // one call of f for both numberings: a second one would cost registers
-        const bool list = act.n >= 0;
-        const int64_t n = list ? (int64_t)act.n * p.mask.bpc : (int64_t)p.n_rows;
-        for (int64_t i = warp0; i < n; i += p.stride) {
-            int64_t r = i;
-            if (list) {
-                const int32_t q = (int32_t)i / p.mask.bpc;
-                r = (int64_t)act.cp[q] * p.mask.bpc + ((int32_t)i - q * p.mask.bpc);
-            } else if (!row_needed(p.mask, r)) {
-                continue;
-            }
-            f(r);
-        }
-        return;
-    }
-    const int64_t n_items = (int64_t)__ldg(p.mask.woff + p.mask.nseg);
-    for (int64_t c0 = warp0 * WIN_RUN; c0 < n_items; c0 += p.stride * WIN_RUN) {
-        int lo = 0, hi = p.mask.nseg; // woff[lo] <= c0 < woff[hi]
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (__ldg(p.mask.woff + mid) <= c0) lo = mid;
-            else hi = mid;
-        }
-        int64_t seg_end = __ldg(p.mask.woff + lo + 1);
-        int64_t r = (int64_t)lo * p.mask.n_cols + __ldg(p.mask.win + lo).x + (c0 - __ldg(p.mask.woff + lo));
-        const int64_t c1 = min(c0 + WIN_RUN, n_items);
-        for (int64_t i = c0; i < c1; ++i, ++r) {
-            while (i == seg_end) { // the next segment with a row (empty windows have none)
-                ++lo;
-                seg_end = __ldg(p.mask.woff + lo + 1);
-                r = (int64_t)lo * p.mask.n_cols + __ldg(p.mask.win + lo).x;
-            }
-            f(r);
-        }
-    }
-}
 
 // The active CPs in ascending order (the whole block, once per launch: a flag per thread and
 // load, ballots, the warps' counts in order).
 template <int THREADS> __device__ __forceinline__ void active_cps(const RowParams &p, ActiveCps &act) {
     const int lane = threadIdx.x & 31;
-    const int K = p.mask.cp_active && !p.mask.win ? p.n_rows / max(p.mask.bpc, 1) : ACT_MAX + 1;
-    if (K > ACT_MAX) { // block-uniform
-        if (threadIdx.x == 0) act.n = -1;
-        __syncthreads();
-        return;
-    }
+    const int K = p.n_rows / max(p.mask.bpc, 1); // at most ACT_MAX
     for (int k0 = 0; k0 < ACT_MAX; k0 += THREADS) {
         const int k = k0 + threadIdx.x;
         const unsigned m = __ballot_sync(0xffffffffu, k < K && p.mask.cp_active[min(k, K - 1)]);
@@ -713,75 +722,108 @@ template <int THREADS> __device__ __forceinline__ void active_cps(const RowParam
     __syncthreads();
 }
 
-template <int THREADS, int UNROLL, typename VT>
+// f over the rows of warp warp0.
+template <int NUM, typename F>
+__device__ __forceinline__ void for_rows(const RowParams &p, const ActiveCps *act, uint32_t warp0, F &&f) {
+    // 32-bit counts throughout: rows are int32, and a count past the last row by one stride stays
+    // below 2^32 (64-bit ones were what the 32-register kernels spilled)
+    [[maybe_unused]] const uint32_t stride = (uint32_t)p.stride;
+    if constexpr (NUM == ROWS_CPS) {
+        // row `at` of active CP number q; a stride is step_cps CPs and step_rows rows (divided by the
+        // host: a reciprocal kept across f costs registers)
+        const uint32_t bpc = (uint32_t)p.mask.bpc;
+        uint32_t q = warp0 / bpc, at = warp0 - q * bpc;
+        while (q < (uint32_t)act->n) {
+            f((int32_t)(act->cp[q] * bpc + at));
+            q += p.step_cps;
+            at += p.step_rows;
+            if (at >= bpc) {
+                at -= bpc;
+                ++q;
+            }
+        }
+    } else if constexpr (NUM == ROWS_ALL) {
+        for (uint32_t r = warp0; r < (uint32_t)p.n_rows; r += stride)
+            if (row_needed(p.mask, r)) f((int32_t)r);
+    } else {
+        // (the item, its row and its segment's end are all that lives across f: the 32-register
+        // kernels have room for no more)
+        const int32_t *woff = p.mask.woff;
+        uint32_t i = warp0 * WIN_RUN, seg_end = 0;
+        int32_t r = 0;
+        while (true) {
+            if (i % WIN_RUN == 0) { // a run starts
+                if (i >= (uint32_t)*(const volatile int32_t *)(woff + p.mask.nseg)) break;
+                int lo = 0, hi = p.mask.nseg; // woff[lo] <= i < woff[hi]
+                while (hi - lo > 1) {
+                    const int mid = (lo + hi) >> 1;
+                    if ((uint32_t)__ldg(woff + mid) <= i) lo = mid;
+                    else hi = mid;
+                }
+                seg_end = (uint32_t)__ldg(woff + hi);
+                r = lo * p.mask.n_cols + __ldg(p.mask.win + lo).x + ((int32_t)i - __ldg(woff + lo));
+            } else if (i == seg_end) { // the next segment with a row (empty windows have none)
+                int lo = (r - 1) / p.mask.n_cols;
+                while (++lo < p.mask.nseg && i == (seg_end = (uint32_t)__ldg(woff + lo + 1))) {}
+                if (lo >= p.mask.nseg) break; // the list's last item has been passed
+                r = lo * p.mask.n_cols + __ldg(p.mask.win + lo).x;
+            }
+            f(r);
+            ++r;
+            ++i;
+            if (i % WIN_RUN == 0) i += (stride - 1) * WIN_RUN;
+        }
+    }
+}
+
+// The body of every warp-row kernel: row_sum(r, lane, pol) is the row's sum, the same in all lanes.
+template <int NUM, int THREADS, typename S>
+__device__ __forceinline__ void warp_rows(const RowParams &p, S &&row_sum) {
+    if (p.skip && *p.skip) return;
+    const ActiveCps *act = nullptr;
+    if constexpr (NUM == ROWS_CPS) {
+        __shared__ ActiveCps list;
+        active_cps<THREADS>(p, list);
+        act = &list;
+    }
+    const int lane = threadIdx.x & 31;
+    const uint32_t warp0 = (blockIdx.x * THREADS + threadIdx.x) >> 5;
+    if (warp0 >= p.stride) return; // warp-uniform, after the block's barriers
+    const uint64_t pol = l2_evict_first_policy();
+    for_rows<NUM>(p, act, warp0, [&](int32_t r) {
+        float sum = row_sum(r, lane, pol);
+        if (lane == 0) {
+            if (p.row_scale) sum *= p.row_scale[r];
+            p.y[p.row_ids ? p.row_ids[r] : r] = sum;
+        }
+    });
+}
+
+template <int NUM, int THREADS, int UNROLL, typename VT>
 __global__ void __launch_bounds__(THREADS) spmv_warp_row_z_kernel(RowParams p) {
-    if (p.skip && *p.skip) return;
-    __shared__ ActiveCps act;
-    active_cps<THREADS>(p, act);
-    const int lane = threadIdx.x & 31;
-    const int64_t warp0 = ((int64_t)blockIdx.x * THREADS + threadIdx.x) >> 5;
-    if (warp0 >= p.stride) return; // warp-uniform, after the block's barriers
-    const uint64_t pol = l2_evict_first_policy();
-    for_rows(p, act, warp0, [&](int64_t r) {
-        float sum = warp_row_sum_z<UNROLL, VT>(p.rowptr, p.cptr, p.cbase, p.col16, p.val, p.x, r, lane, pol);
-        if (lane == 0) {
-            if (p.row_scale) sum *= p.row_scale[r];
-            p.y[p.row_ids ? p.row_ids[r] : r] = sum;
-        }
+    warp_rows<NUM, THREADS>(p, [&](int32_t r, int lane, uint64_t pol) {
+        return warp_row_sum_z<UNROLL, VT>(p.rowptr, p.cptr, p.cbase, p.col16, p.val, p.x, r, lane, pol);
     });
 }
 
-template <int THREADS, int CTAS, typename VT>
+template <int NUM, int THREADS, int CTAS, typename VT>
 __global__ void __launch_bounds__(THREADS, CTAS) spmv_warp_row_x_kernel(RowParams p) {
-    if (p.skip && *p.skip) return;
-    __shared__ ActiveCps act;
-    active_cps<THREADS>(p, act);
-    const int lane = threadIdx.x & 31;
-    const int64_t warp0 = ((int64_t)blockIdx.x * THREADS + threadIdx.x) >> 5;
-    if (warp0 >= p.stride) return; // warp-uniform, after the block's barriers
-    const uint64_t pol = l2_evict_first_policy();
-    for_rows(p, act, warp0, [&](int64_t r) {
-        float sum = warp_row_sum_x<VT>(p.rowptr, p.col, p.strm, p.sptr, p.x, r, lane, pol);
-        if (lane == 0) {
-            if (p.row_scale) sum *= p.row_scale[r];
-            p.y[p.row_ids ? p.row_ids[r] : r] = sum;
-        }
+    warp_rows<NUM, THREADS>(p, [&](int32_t r, int lane, uint64_t pol) {
+        return warp_row_sum_x<VT>(p.rowptr, p.col, p.strm, p.sptr, p.x, r, lane, pol);
     });
 }
 
-template <int THREADS, int UNROLL, typename VT>
+template <int NUM, int THREADS, int UNROLL, typename VT>
 __global__ void __launch_bounds__(THREADS) spmv_warp_row_c_kernel(RowParams p) {
-    if (p.skip && *p.skip) return;
-    __shared__ ActiveCps act;
-    active_cps<THREADS>(p, act);
-    const int lane = threadIdx.x & 31;
-    const int64_t warp0 = ((int64_t)blockIdx.x * THREADS + threadIdx.x) >> 5;
-    if (warp0 >= p.stride) return; // warp-uniform, after the block's barriers
-    const uint64_t pol = l2_evict_first_policy();
-    for_rows(p, act, warp0, [&](int64_t r) {
-        float sum = warp_row_sum_c<UNROLL, VT>(p.rowptr, p.col, p.val, p.x, r, lane, pol);
-        if (lane == 0) {
-            if (p.row_scale) sum *= p.row_scale[r];
-            p.y[p.row_ids ? p.row_ids[r] : r] = sum;
-        }
+    warp_rows<NUM, THREADS>(p, [&](int32_t r, int lane, uint64_t pol) {
+        return warp_row_sum_c<UNROLL, VT>(p.rowptr, p.col, p.val, p.x, r, lane, pol);
     });
 }
 
-template <int THREADS, int UNROLL, typename VT>
+template <int NUM, int THREADS, int UNROLL, typename VT>
 __global__ void __launch_bounds__(THREADS) spmv_warp_row_kernel(RowParams p) {
-    if (p.skip && *p.skip) return;
-    __shared__ ActiveCps act;
-    active_cps<THREADS>(p, act);
-    const int lane = threadIdx.x & 31;
-    const int64_t warp0 = ((int64_t)blockIdx.x * THREADS + threadIdx.x) >> 5;
-    if (warp0 >= p.stride) return; // warp-uniform, after the block's barriers
-    const uint64_t pol = l2_evict_first_policy();
-    for_rows(p, act, warp0, [&](int64_t r) {
-        float sum = warp_row_sum<UNROLL, VT>(p.rowptr, p.col, p.val, p.x, r, lane, pol);
-        if (lane == 0) {
-            if (p.row_scale) sum *= p.row_scale[r];
-            p.y[p.row_ids ? p.row_ids[r] : r] = sum;
-        }
+    warp_rows<NUM, THREADS>(p, [&](int32_t r, int lane, uint64_t pol) {
+        return warp_row_sum<UNROLL, VT>(p.rowptr, p.col, p.val, p.x, r, lane, pol);
     });
 }
 
@@ -944,29 +986,29 @@ template <typename VT> TileFn tile_kernel_for(int cfg) {
     }
 }
 
-template <typename VT> RowFn row_kernel_for(int cfg) {
+template <int NUM, typename VT> RowFn row_kernel_for(int cfg) {
     switch (cfg) {
-    case 4: return spmv_warp_row_kernel<256, 2, VT>;
-    case 5: return spmv_warp_row_kernel<256, 1, VT>;
-    case 7: return spmv_warp_row_kernel<256, 4, VT>;
-    case 8: return spmv_warp_row_kernel<256, 8, VT>;
-    case 9: return spmv_warp_row_c_kernel<256, 4, VT>;
-    case 10: return spmv_warp_row_c_kernel<256, 8, VT>;
-    case 11: return spmv_warp_row_c_kernel<512, 4, VT>;
-    case 12: return spmv_warp_row_z_kernel<256, 4, VT>;
-    case 13: return spmv_warp_row_z_kernel<256, 8, VT>;
-    case 14: return spmv_warp_row_z_kernel<512, 4, VT>;
-    default: return spmv_warp_row_kernel<512, 4, VT>;
+    case 4: return spmv_warp_row_kernel<NUM, 256, 2, VT>;
+    case 5: return spmv_warp_row_kernel<NUM, 256, 1, VT>;
+    case 7: return spmv_warp_row_kernel<NUM, 256, 4, VT>;
+    case 8: return spmv_warp_row_kernel<NUM, 256, 8, VT>;
+    case 9: return spmv_warp_row_c_kernel<NUM, 256, 4, VT>;
+    case 10: return spmv_warp_row_c_kernel<NUM, 256, 8, VT>;
+    case 11: return spmv_warp_row_c_kernel<NUM, 512, 4, VT>;
+    case 12: return spmv_warp_row_z_kernel<NUM, 256, 4, VT>;
+    case 13: return spmv_warp_row_z_kernel<NUM, 256, 8, VT>;
+    case 14: return spmv_warp_row_z_kernel<NUM, 512, 4, VT>;
+    default: return spmv_warp_row_kernel<NUM, 512, 4, VT>;
     }
 }
 
 // The stream's kernel for a consecutive-lane configuration: 256 threads with 8 or 6 CTAs per
 // SM (32 or 40 registers), 512 with 4.  The autotuner times them as it times the others.
-template <typename VT> RowFn stream_kernel_for(int cfg) {
+template <int NUM, typename VT> RowFn stream_kernel_for(int cfg) {
     switch (cfg) {
-    case 9: return spmv_warp_row_x_kernel<256, 8, VT>;
-    case 10: return spmv_warp_row_x_kernel<256, 6, VT>;
-    default: return spmv_warp_row_x_kernel<512, 4, VT>;
+    case 9: return spmv_warp_row_x_kernel<NUM, 256, 8, VT>;
+    case 10: return spmv_warp_row_x_kernel<NUM, 256, 6, VT>;
+    default: return spmv_warp_row_x_kernel<NUM, 512, 4, VT>;
     }
 }
 
@@ -980,49 +1022,53 @@ template <typename VT> int smem_for(int cfg) {
     }
 }
 
+// The kernel of a configuration for one form of the matrix (CSR or packed stream) and one numbering.
 struct Launch {
     TileFn tile = nullptr;
     RowFn row = nullptr;
-    RowFn strm = nullptr; // the same configuration reading the packed stream
-    int threads = 0, smem = 0, blocks_per_sm = 0, blocks_strm = 0;
+    int threads = 0, smem = 0, blocks_per_sm = 0;
 };
 
-template <typename VT> static void pick(int cfg, Launch &n) {
+template <int NUM, typename VT> static void pick(int cfg, bool strm, Launch &n) {
     if (kCfgs[cfg].family == 0) {
         n.tile = tile_kernel_for<VT>(cfg);
         n.smem = smem_for<VT>(cfg);
     } else {
-        n.row = row_kernel_for<VT>(cfg);
-        if (kCfgs[cfg].family == 2) n.strm = stream_kernel_for<VT>(cfg);
-        n.smem = 0;
+        n.row = strm ? stream_kernel_for<NUM, VT>(cfg) : row_kernel_for<NUM, VT>(cfg);
     }
 }
+template <typename VT> static void pick(int cfg, bool strm, Numbering num, Launch &n) {
+    if (num == ROWS_WINDOWS) pick<ROWS_WINDOWS, VT>(cfg, strm, n);
+    else if (num == ROWS_CPS) pick<ROWS_CPS, VT>(cfg, strm, n);
+    else pick<ROWS_ALL, VT>(cfg, strm, n);
+}
 
-static vmat_status launch_info(vmat_dtype dt, int cfg, Launch *out) {
-    static Launch cache[3][N_CFG];
-    static int cached_dev[3][N_CFG];
+static vmat_status launch_info(vmat_dtype dt, int cfg, bool strm, Numbering num, Launch *out) {
+    static std::mutex mu;
+    static Launch cache[3][N_CFG][2][N_NUMBERINGS];
+    static int cached_dev[3][N_CFG][2][N_NUMBERINGS];
     int dev;
     VMAT_CUDA(cudaGetDevice(&dev));
-    Launch &L = cache[dt][cfg];
-    if ((L.tile || L.row) && cached_dev[dt][cfg] == dev) {
+    std::lock_guard<std::mutex> lock(mu);
+    Launch &L = cache[dt][cfg][strm][num];
+    if ((L.tile || L.row) && cached_dev[dt][cfg][strm][num] == dev) {
         *out = L;
         return VMAT_OK;
     }
     Launch n;
     n.threads = kCfgs[cfg].threads;
-    if (dt == VMAT_F32) pick<float>(cfg, n);
-    else if (dt == VMAT_BF16) pick<__nv_bfloat16>(cfg, n);
-    else pick<__nv_fp8_e4m3>(cfg, n);
+    if (dt == VMAT_F32) pick<float>(cfg, strm, num, n);
+    else if (dt == VMAT_BF16) pick<__nv_bfloat16>(cfg, strm, num, n);
+    else pick<__nv_fp8_e4m3>(cfg, strm, num, n);
     if (n.tile) {
         VMAT_CUDA(cudaFuncSetAttribute(n.tile, cudaFuncAttributeMaxDynamicSharedMemorySize, n.smem));
         VMAT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n.blocks_per_sm, n.tile, n.threads, n.smem));
     } else {
         VMAT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n.blocks_per_sm, n.row, n.threads, 0));
-        if (n.strm) VMAT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n.blocks_strm, n.strm, n.threads, 0));
     }
     if (n.blocks_per_sm < 1) return set_error(VMAT_ECUDA, "spmv: configuration %d does not fit on an SM", cfg);
     L = n;
-    cached_dev[dt][cfg] = dev;
+    cached_dev[dt][cfg][strm][num] = dev;
     *out = n;
     return VMAT_OK;
 }
@@ -1075,8 +1121,9 @@ vmat_status spmv_run(const Ddc &h, const CsrMat &m, const float *x, float *y, co
                      cudaStream_t s, const int32_t *skip) {
     DeviceCtx *ctx;
     VMAT_TRY(device_ctx(&ctx));
+    const bool strm = m.strm && spmv_config_stream(m.cfg);
     Launch L;
-    VMAT_TRY(launch_info(h.dtype, m.cfg, &L));
+    VMAT_TRY(launch_info(h.dtype, m.cfg, strm, numbering_of(mask, m.n_rows), &L));
     if (L.row) {
         RowParams p;
         p.rowptr = m.rowptr;
@@ -1089,7 +1136,6 @@ vmat_status spmv_run(const Ddc &h, const CsrMat &m, const float *x, float *y, co
         p.mask = mask;
         p.n_rows = m.n_rows;
         p.skip = skip;
-        const bool strm = L.strm && m.strm && L.blocks_strm > 0;
         p.strm = m.strm;
         p.sptr = m.sptr;
         p.col16 = m.col16;
@@ -1099,11 +1145,12 @@ vmat_status spmv_run(const Ddc &h, const CsrMat &m, const float *x, float *y, co
             return set_error(VMAT_ESTATE, "spmv: configuration %d needs the 16-bit column index", m.cfg);
         const int64_t warps = std::max<int64_t>(1, m.n_rows);
         const int64_t want = (warps * 32 + L.threads - 1) / L.threads;
-        const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)ctx->n_sm * (strm ? L.blocks_strm
-                                                                                                             : L.blocks_per_sm)));
+        const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)ctx->n_sm * L.blocks_per_sm));
         const int64_t n_warps = (int64_t)grid * L.threads / 32;
         p.stride = mask.win && !mask.woff ? coprime_stride(n_warps, &mask.n_cols, 1) : n_warps;
-        (strm ? L.strm : L.row)<<<grid, L.threads, 0, s>>>(p);
+        p.step_cps = (uint32_t)(p.stride / std::max(mask.bpc, 1));
+        p.step_rows = (uint32_t)(p.stride % std::max(mask.bpc, 1));
+        L.row<<<grid, L.threads, 0, s>>>(p);
         VMAT_LAUNCH_CHECK();
         return VMAT_OK;
     }
