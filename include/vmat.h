@@ -224,6 +224,10 @@ vmat_status ddc_free(vmat_ddc h);
 /* Sizes and build facts of a handle (host struct). */
 vmat_status ddc_info(vmat_ddc h, vmat_ddc_info *out);
 
+/* Device bytes of each CSR's packed stream (build option autotune, configurations 9-11), 0 where
+ * the handle holds none.  They come on top of vmat_ddc_info's bytes_D and bytes_Dt. */
+vmat_status vmat_ddc_stream_bytes(vmat_ddc h, int64_t *bytes_D, int64_t *bytes_Dt);
+
 /* ---- Sparse products (hot path) ------------------------------------------ */
 
 /* d = D x (Section 2.1: z_i = sum_j D_ij x_j; Eq. 5 is the case x = the

@@ -136,6 +136,13 @@ def ddc_info(h: int) -> dict:
     return {f: getattr(info, f) for f, _ in info._fields_}
 
 
+def ddc_stream_bytes(h: int) -> tuple:
+    """Device bytes of the packed streams of CSR(D) and CSR(D^T), 0 where the handle holds none."""
+    d, dt = ctypes.c_int64(), ctypes.c_int64()
+    check("vmat_ddc_stream_bytes", _lib.load().vmat_ddc_stream_bytes(ctypes.c_void_p(h), ctypes.byref(d), ctypes.byref(dt)))
+    return d.value, dt.value
+
+
 # ---------------------------------------------------------------------------- products
 
 def dose_forward(h: int, x: torch.Tensor, d: torch.Tensor, stream=None) -> None:

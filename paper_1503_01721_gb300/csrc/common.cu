@@ -359,4 +359,17 @@ vmat_status ddc_info(vmat_ddc hd, vmat_ddc_info *out) {
     return VMAT_OK;
 }
 
+vmat_status vmat_ddc_stream_bytes(vmat_ddc hd, int64_t *bytes_D, int64_t *bytes_Dt) {
+    clear_error();
+    if (!hd || !bytes_D || !bytes_Dt) return set_error(VMAT_EINVAL, "vmat_ddc_stream_bytes: NULL argument");
+    const Ddc *h = as_ddc(hd);
+    const int vb = value_bytes(h->dtype);
+    auto bytes = [&](const CsrMat &m) {
+        return m.strm ? m.strm_recs * strm_record_bytes(vb) + ((int64_t)m.n_rows + 1) * 4 : (int64_t)0;
+    };
+    *bytes_D = bytes(h->D);
+    *bytes_Dt = bytes(h->Dt);
+    return VMAT_OK;
+}
+
 } // extern "C"

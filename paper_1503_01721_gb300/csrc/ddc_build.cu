@@ -776,6 +776,7 @@ vmat_status csr_build_stream(CsrMat &m, int vb, int n_sm, cudaStream_t s) {
     VMAT_CUDA(cudaStreamSynchronize(s));
     if (n_far * 16 > (unsigned long long)n_rec * (STRM_ENTRIES / 32)) return VMAT_OK;
     m.strm = (unsigned char *)b_strm.release();
+    m.strm_recs = n_rec;
     m.sptr = (int32_t *)b_sptr.release();
     return VMAT_OK;
 }

@@ -107,6 +107,7 @@ struct CsrMat {
     // The matrix once more as a packed stream for the consecutive-lane configurations (null:
     // they read col and val): see csr_build_stream.
     unsigned char *strm = nullptr; // [strm_recs] records
+    int64_t strm_recs = 0;
     int32_t *sptr = nullptr;       // [n_rows + 1] first record of each row
     // tiles
     int cfg = 0;                 // tile configuration index

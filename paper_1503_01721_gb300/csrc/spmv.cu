@@ -1322,6 +1322,7 @@ vmat_status spmv_autotune(Ddc &h, cudaStream_t s) {
             cudaFree(m->sptr);
             m->strm = nullptr;
             m->sptr = nullptr;
+            m->strm_recs = 0;
         }
     }
     VMAT_CUDA(cudaStreamSynchronize(s));
