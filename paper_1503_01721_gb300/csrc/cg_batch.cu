@@ -107,6 +107,7 @@ struct Batch {
     int64_t device_bytes = 0;
     SpmvPlan *d_spmv = nullptr;
     int64_t *d_rows_off = nullptr, tot_rows = 0;
+    int32_t n_strm = 0; // plans whose CSR(D^T) holds a packed stream
     PricePlan *d_price = nullptr;
     int64_t *d_price_off = nullptr, tot_price = 0;
     int32_t max_cols = 1;
@@ -178,7 +179,7 @@ static vmat_status enqueue_run(Batch &b, cudaStream_t s) {
         VMAT_LAUNCH_CHECK();
         VMAT_TRY(objective_grad_batched(b.d_obj, b.d_na_off, n, b.tot_na, s));
         VMAT_TRY(price_windows_batched(b.d_win, n, b.max_K, t, s));
-        VMAT_TRY(spmv_rows_batched(b.dt, b.spmv_cfg, b.d_spmv, b.d_rows_off, n, b.tot_rows, s, b.cols.data(),
+        VMAT_TRY(spmv_rows_batched(b.dt, b.spmv_cfg, b.d_spmv, b.d_rows_off, n, b.n_strm, b.tot_rows, s, b.cols.data(),
                                    (int)b.cols.size()));
         VMAT_TRY(price_apertures_batched(b.d_price, b.d_price_off, n, b.tot_price, b.max_cols, s));
         if (b.any_interdig) // the chain DP over rows (Section 2.2.2), each such plan on its own scratch
@@ -351,6 +352,7 @@ static vmat_status make_batch(Batch &b, int32_t n_plans, const vmat_plan_desc *p
         const bool fp8 = h.dtype == VMAT_FP8E4M3;
         spmv[i] = SpmvPlan{h.Dt.rowptr, h.Dt.col, h.Dt.val, h.Dt.strm, h.Dt.sptr, p.g_full, p.pi, fp8 ? h.scale : nullptr, nullptr,
                            RowMask{nullptr, p.win, p.bpc, p.mlc.n_cols}, p.ctl, h.Dt.n_rows};
+        b.n_strm += h.Dt.strm ? 1 : 0;
         PricePlan &q = price[i];
         VMAT_TRY(pricing_geom(&p.mlc, &q.g));
         wins[i] = WinPlan{q.g, p.occupied, p.leaves_all, p.win, h.Dt.rowptr, p.wcount, p.ctl};
@@ -468,10 +470,10 @@ static vmat_status make_batch(Batch &b, int32_t n_plans, const vmat_plan_desc *p
         float best = 1e30f;
         for (int cfg = 0; cfg < spmv_n_configs() && cfg < 32; ++cfg) {  // warp-row families only
             if (!spmv_batched_config(cfg)) continue;
-            VMAT_TRY(spmv_rows_batched(b.dt, cfg, b.d_spmv, b.d_rows_off, n_plans, b.tot_rows, s, b.cols.data(),
+            VMAT_TRY(spmv_rows_batched(b.dt, cfg, b.d_spmv, b.d_rows_off, n_plans, b.n_strm, b.tot_rows, s, b.cols.data(),
                                        (int)b.cols.size())); // warm-up
             VMAT_CUDA(cudaEventRecord(e0, s));
-            VMAT_TRY(spmv_rows_batched(b.dt, cfg, b.d_spmv, b.d_rows_off, n_plans, b.tot_rows, s, b.cols.data(),
+            VMAT_TRY(spmv_rows_batched(b.dt, cfg, b.d_spmv, b.d_rows_off, n_plans, b.n_strm, b.tot_rows, s, b.cols.data(),
                                        (int)b.cols.size()));
             VMAT_CUDA(cudaEventRecord(e1, s));
             VMAT_CUDA(cudaEventSynchronize(e1));

@@ -412,8 +412,9 @@ vmat_status price_apertures_batched(const PricePlan *plans, const int64_t *off, 
                                     int32_t max_cols, cudaStream_t s);
 // cols (host, may be null): the plans' MLC column counts (n_cols entries); the row
 // stride is chosen coprime with each so that windowed passes stay balanced.
+// n_strm: how many of the plans' matrices hold a packed stream.
 vmat_status spmv_rows_batched(vmat_dtype dt, int cfg, const SpmvPlan *plans, const int64_t *row_off, int32_t n_plans,
-                              int64_t total_rows, cudaStream_t s, const int32_t *cols = nullptr, int n_cols = 0);
+                              int32_t n_strm, int64_t total_rows, cudaStream_t s, const int32_t *cols = nullptr, int n_cols = 0);
 
 // Objective over n voxels.  idx (may be null): voxel i of z is voxel idx[i] of struct_id.
 // g_scatter (may be null): write g[i] to g_scatter[idx[i]] instead of g[i].

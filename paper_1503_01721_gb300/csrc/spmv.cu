@@ -829,40 +829,63 @@ __global__ void __launch_bounds__(THREADS) spmv_warp_row_kernel(RowParams p) {
 
 // Several plans' matrices in one launch: global row g belongs to plan p with
 // row_off[p] <= g < row_off[p + 1] (row g - row_off[p] of that plan).  A warp
-// looks its plan up when it crosses into another plan's range.
-template <int THREADS, int UNROLL, typename VT, bool CONSEC>
-__global__ void __launch_bounds__(THREADS)
+// looks its plan up when it crosses into another plan's range, and keeps it in shared memory: a
+// plan's pointers in registers (64-128 of them) left room for half as many warps as the
+// single-plan kernels hold.  Best configuration of the four plans below, in ms: from the CSR with the plan in
+// registers -> the same with either form read in one kernel -> now: FP32 0.335 -> 0.335 -> 0.244,
+// BF16 0.339 -> 0.352 -> 0.193, FP8 0.320 -> 0.308 -> 0.214.
+// FORM: what the plans' rows are read from, lane-strided chunks of the CSR (configurations 4-8), consecutive
+// lanes of the CSR, the packed stream, or each plan's stream where it holds one and its CSR where not
+// (9-11).  Two row sums in one kernel cost registers, so only a batch of both kinds runs BATCH_EITHER.
+enum BatchForm { BATCH_CHUNKS, BATCH_CSR, BATCH_STREAM, BATCH_EITHER };
+struct WarpPlan {
+    SpmvPlan P;
+    int64_t lo, hi; // the plan's global rows
+    int skip;
+};
+template <int THREADS, int CTAS, int UNROLL, typename VT, BatchForm FORM>
+__global__ void __launch_bounds__(THREADS, CTAS)
     spmv_rows_batched_kernel(const SpmvPlan *__restrict__ plans, const int64_t *__restrict__ row_off, int32_t n_plans,
                              int64_t total_rows, int64_t stride) {
     __shared__ int64_t soff[VMAT_MAX_BATCH + 1];
+    __shared__ WarpPlan wplan[THREADS / 32];
+    static_assert(sizeof(SpmvPlan) % 4 == 0, "copied in words");
     for (int i = threadIdx.x; i <= n_plans; i += THREADS) soff[i] = row_off[i];
-    __syncthreads();
     const int lane = threadIdx.x & 31;
+    WarpPlan &W = wplan[threadIdx.x >> 5];
+    if (lane == 0) W.lo = W.hi = 0;
+    __syncthreads();
     const int64_t warp0 = ((int64_t)blockIdx.x * THREADS + threadIdx.x) >> 5;
     if (warp0 >= stride) return; // warp-uniform, after the block's only barrier
     const uint64_t pol = l2_evict_first_policy();
-    int64_t lo = 0, hi = 0;
-    SpmvPlan P;
-    bool skip = true;
     for (int64_t gr = warp0; gr < total_rows; gr += stride) {
-        if (gr < lo || gr >= hi) {
+        if (gr < W.lo || gr >= W.hi) {
             int a = 0, b = n_plans; // soff[a] <= gr < soff[b]
             while (b - a > 1) {
                 const int m = (a + b) >> 1;
                 if (soff[m] <= gr) a = m;
                 else b = m;
             }
-            P = plans[a];
-            lo = soff[a];
-            hi = soff[a + 1];
-            skip = P.skip && *P.skip;
+            __syncwarp();
+            const uint32_t *src = reinterpret_cast<const uint32_t *>(plans + a);
+            for (int i = lane; i < (int)(sizeof(SpmvPlan) / 4); i += 32) reinterpret_cast<uint32_t *>(&W.P)[i] = src[i];
+            __syncwarp();
+            if (lane == 0) {
+                W.lo = soff[a];
+                W.hi = soff[a + 1];
+                W.skip = W.P.skip && *W.P.skip;
+            }
+            __syncwarp();
         }
-        if (skip) continue;
-        const int64_t r = gr - lo;
-        if (!row_needed(P.mask, r)) continue;
-        float sum = !CONSEC  ? warp_row_sum<UNROLL, VT>(P.rowptr, P.col, P.val, P.x, r, lane, pol)
-                    : P.strm ? warp_row_sum_x<VT>(P.rowptr, P.col, P.strm, P.sptr, P.x, r, lane, pol)
-                             : warp_row_sum_c<UNROLL, VT>(P.rowptr, P.col, P.val, P.x, r, lane, pol);
+        if (W.skip) continue;
+        const int32_t r = (int32_t)(gr - W.lo);
+        if (!row_needed(W.P.mask, r)) continue;
+        const SpmvPlan &P = W.P;
+        float sum;
+        if (FORM == BATCH_CHUNKS) sum = warp_row_sum<UNROLL, VT>(P.rowptr, P.col, P.val, P.x, r, lane, pol);
+        else if (FORM == BATCH_STREAM || (FORM == BATCH_EITHER && P.strm))
+            sum = warp_row_sum_x<VT>(P.rowptr, P.col, P.strm, P.sptr, P.x, r, lane, pol);
+        else sum = warp_row_sum_c<UNROLL, VT>(P.rowptr, P.col, P.val, P.x, r, lane, pol);
         if (lane == 0) {
             if (P.row_scale) sum *= P.row_scale[r];
             P.y[P.row_ids ? P.row_ids[r] : r] = sum;
@@ -1195,17 +1218,35 @@ vmat_status spmv_run(const Ddc &h, const CsrMat &m, const float *x, float *y, co
     return VMAT_OK;
 }
 
-template <typename VT> static RowBatchFn batched_kernel_for(int cfg) {
+template <typename VT, BatchForm FORM> static RowBatchFn batched_consecutive_for(int cfg) {
     switch (cfg) {
-    case 4: return spmv_rows_batched_kernel<256, 2, VT, false>;
-    case 5: return spmv_rows_batched_kernel<256, 1, VT, false>;
-    case 6: return spmv_rows_batched_kernel<512, 4, VT, false>;
-    case 7: return spmv_rows_batched_kernel<256, 4, VT, false>;
-    case 8: return spmv_rows_batched_kernel<256, 8, VT, false>;
-    case 9: return spmv_rows_batched_kernel<256, 4, VT, true>;
-    case 10: return spmv_rows_batched_kernel<256, 8, VT, true>;
-    case 11: return spmv_rows_batched_kernel<512, 4, VT, true>;
-    default: return nullptr;
+    case 9: return spmv_rows_batched_kernel<256, 1, 4, VT, FORM>;
+    case 10: return spmv_rows_batched_kernel<256, 1, 8, VT, FORM>;
+    default: return spmv_rows_batched_kernel<512, 1, 4, VT, FORM>;
+    }
+}
+// Registers of the stream's batched kernels: 40 (48 for configuration 10), since at 32 the plan's
+// pointers and the row counts spill a few words.  BF16 at 512 threads takes the 32 registers and
+// 64 warps all the same: four plans of 80 x 80 x 60 voxels and 45 CPs down to 51 x 51 x 38 and 31,
+// 0.193 ms instead of 0.300 (FP32 0.257 instead of 0.244, FP8 0.228 instead of 0.214).
+template <typename VT> static RowBatchFn batched_stream_for(int cfg) {
+    switch (cfg) {
+    case 9: return spmv_rows_batched_kernel<256, 6, 1, VT, BATCH_STREAM>;
+    case 10: return spmv_rows_batched_kernel<256, 5, 1, VT, BATCH_STREAM>;
+    default: return spmv_rows_batched_kernel<512, sizeof(VT) == 2 ? 4 : 3, 1, VT, BATCH_STREAM>;
+    }
+}
+template <typename VT> static RowBatchFn batched_kernel_for(int cfg, int n_plans, int n_strm) {
+    switch (cfg) {
+    case 4: return spmv_rows_batched_kernel<256, 1, 2, VT, BATCH_CHUNKS>;
+    case 5: return spmv_rows_batched_kernel<256, 1, 1, VT, BATCH_CHUNKS>;
+    case 6: return spmv_rows_batched_kernel<512, 1, 4, VT, BATCH_CHUNKS>;
+    case 7: return spmv_rows_batched_kernel<256, 1, 4, VT, BATCH_CHUNKS>;
+    case 8: return spmv_rows_batched_kernel<256, 1, 8, VT, BATCH_CHUNKS>;
+    default:
+        return n_strm == 0         ? batched_consecutive_for<VT, BATCH_CSR>(cfg)
+               : n_strm == n_plans ? batched_stream_for<VT>(cfg)
+                                   : batched_consecutive_for<VT, BATCH_EITHER>(cfg);
     }
 }
 
@@ -1214,15 +1255,15 @@ bool spmv_batched_config(int cfg) {
 }
 
 vmat_status spmv_rows_batched(vmat_dtype dt, int cfg, const SpmvPlan *plans, const int64_t *row_off, int32_t n_plans,
-                              int64_t total_rows, cudaStream_t s, const int32_t *cols, int n_cols) {
+                              int32_t n_strm, int64_t total_rows, cudaStream_t s, const int32_t *cols, int n_cols) {
     if (!spmv_batched_config(cfg)) return set_error(VMAT_EINVAL, "spmv_rows_batched: configuration %d is not warp-row", cfg);
     if (n_plans < 1 || n_plans > VMAT_MAX_BATCH) return set_error(VMAT_EINVAL, "spmv_rows_batched: bad plan count");
     if (total_rows <= 0) return VMAT_OK;
     DeviceCtx *ctx;
     VMAT_TRY(device_ctx(&ctx));
-    RowBatchFn fn = dt == VMAT_F32 ? batched_kernel_for<float>(cfg)
-                    : dt == VMAT_BF16 ? batched_kernel_for<__nv_bfloat16>(cfg)
-                                      : batched_kernel_for<__nv_fp8_e4m3>(cfg);
+    RowBatchFn fn = dt == VMAT_F32 ? batched_kernel_for<float>(cfg, n_plans, n_strm)
+                    : dt == VMAT_BF16 ? batched_kernel_for<__nv_bfloat16>(cfg, n_plans, n_strm)
+                                      : batched_kernel_for<__nv_fp8_e4m3>(cfg, n_plans, n_strm);
     const int threads = kCfgs[cfg].threads;
     int bps = 1;
     VMAT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, fn, threads, 0));

@@ -34,3 +34,12 @@ def test_stream_kernels_spill_nothing(ptxas_lines):
     entries = _spills(ptxas_lines, "spmv_warp_row_x_kernel")
     assert len(entries) >= 9
     assert [e for e in entries if e[1] or e[2]] == []
+
+
+def test_batched_stream_kernels_spill_nothing(ptxas_lines):
+    """Batches whose plans all hold the stream (BF16 at 512 threads apart, which spills a little for
+    twice the warps)."""
+    entries = [e for e in _spills(ptxas_lines, "spmv_rows_batched_kernel") if "BatchFormE2E" in e[0]]
+    assert len(entries) == 9
+    assert len([e for e in entries if e[1] or e[2]]) <= 1
+    assert [e for e in entries if (e[1] or e[2]) and not ("Li512ELi4E" in e[0] and "bfloat16" in e[0])] == []
