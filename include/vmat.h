@@ -102,7 +102,8 @@ typedef struct {
                            and one with a consecutive-lane configuration (9-11), also holds each CSR as
                            a packed stream that those configurations read (records of 128 entries with
                            16-bit column offsets: s_val + 2.1 bytes per entry, rows padded to whole
-                           records; same sums, same bits), where memory allows and the columns of
+                           records; same sums, same bits), where at least half of the device's memory
+                           stays free, rows are long enough to fill records and the columns of
                            nearly every 32 entries span fewer than 65,536 */
     int32_t keep_coo;   /* nonzero: keep the COO copy after the build */
     int32_t index16;    /* nonzero: also store 16-bit column indices (rows cut into 128-entry

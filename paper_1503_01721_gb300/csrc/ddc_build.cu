@@ -756,7 +756,11 @@ vmat_status csr_build_stream(CsrMat &m, int vb, int n_sm, cudaStream_t s) {
     if (n_rec > INT32_MAX) return VMAT_OK;
     // rows of a few entries pad most of a record: such a matrix would read more, not less
     if ((double)n_rec * strm_record_bytes(vb) > (double)m.nnz * (vb + 4)) return VMAT_OK;
-    if (b_strm.alloc((size_t)n_rec * strm_record_bytes(vb)) != cudaSuccess) return skip();
+    size_t mem_free = 0, mem_total = 0;
+    VMAT_CUDA(cudaMemGetInfo(&mem_free, &mem_total));
+    const size_t bytes = (size_t)n_rec * strm_record_bytes(vb);
+    if (mem_free < bytes + mem_total / 2) return VMAT_OK; // what has to fit comes first: other handles, plans, batches
+    if (b_strm.alloc(bytes) != cudaSuccess) return skip();
     narrow_offsets<<<grid_for(m.n_rows + 1, n_sm), BUILD_THREADS, 0, s>>>((int64_t *)b_ptr.p, m.n_rows + 1,
                                                                          (int32_t *)b_sptr.p);
     VMAT_LAUNCH_CHECK();
@@ -1028,7 +1032,6 @@ extern "C" vmat_status ddc_build(vmat_ddc hd, const vmat_build_opts *opts_in, vo
         m.row_ids = nullptr;
         m.max_row = max_row_t;
         if (opts.index16) VMAT_TRY(csr_build_index16(m, n_sm, s));
-        if (opts.autotune || spmv_config_stream(cfg_dt)) VMAT_TRY(csr_build_stream(m, vb, n_sm, s));
         VMAT_TRY(spmv_prepare_tiles(m, cfg_dt, s));
         h->built_Dt = true;
     }
@@ -1057,7 +1060,6 @@ extern "C" vmat_status ddc_build(vmat_ddc hd, const vmat_build_opts *opts_in, vo
         m.row_ids = h->act_vox;
         m.max_row = max_row_d;
         if (opts.index16) VMAT_TRY(csr_build_index16(m, n_sm, s));
-        if (opts.autotune || spmv_config_stream(cfg)) VMAT_TRY(csr_build_stream(m, vb, n_sm, s));
         VMAT_TRY(spmv_prepare_tiles(m, cfg, s));
         h->built_D = true;
     }
@@ -1075,6 +1077,9 @@ extern "C" vmat_status ddc_build(vmat_ddc hd, const vmat_build_opts *opts_in, vo
         h->coo_vox = h->coo_blt = nullptr;
         h->coo_val = nullptr;
     }
+    // the streams last: they may be left out, and what the build and the COO held is free by now
+    if (opts.build_Dt && (opts.autotune || spmv_config_stream(cfg_dt))) VMAT_TRY(csr_build_stream(h->Dt, vb, n_sm, s));
+    if (opts.build_D && (opts.autotune || spmv_config_stream(cfg))) VMAT_TRY(csr_build_stream(h->D, vb, n_sm, s));
     VMAT_CUDA(cudaEventRecord(e1, s));
     VMAT_CUDA(cudaEventSynchronize(e1));
     float ms = 0.f;

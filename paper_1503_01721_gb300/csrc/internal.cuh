@@ -260,7 +260,8 @@ __host__ __device__ constexpr int strm_record_bytes(int vb) { return 16 + STRM_E
 // Is configuration cfg one that reads the packed stream when the matrix holds it?
 bool spmv_config_stream(int cfg);
 // Builds m.strm / m.sptr from m.col and m.val (vb bytes per value).  VMAT_OK without it when
-// memory is short or when more than 1/16 of the 32-entry chunks span 65,536 columns.
+// less than half of the device's memory would stay free, when the rows are so short that it would
+// hold more bytes than the CSR or when more than 1/16 of the 32-entry chunks span 65,536 columns.
 vmat_status csr_build_stream(CsrMat &m, int vb, int n_sm, cudaStream_t s);
 // Builds m.col16 / cbase / cptr when every chunk fits 16 bits (else leaves them null).
 vmat_status csr_build_index16(CsrMat &m, int n_sm, cudaStream_t s);

@@ -163,3 +163,28 @@ def test_a_refused_stream_leaves_the_csr(rows, why):
     bound = spmv_bound(abs(D).T @ np.abs(g.astype(np.float64)), np.bincount(blt, minlength=J))
     for pi in out:
         assert np.all(np.abs(pi - oracle.beamlet_price(D, g)) <= bound)
+
+
+def test_the_stream_gives_way_when_memory_is_short():
+    """With less than half of the device's memory left a build takes no stream, and its products are
+    the CSR's: the stream is optional, what a later build or plan allocates is not."""
+    from paper_1503_01721_gb300 import api
+    c = synth.make_case("cfg1", seed=0)
+    g = dev(synth.random_vector(c.V, 1), torch.float32)
+    out = []
+    _, total = torch.cuda.mem_get_info()
+    for held in (int(0.55 * total), 0):
+        block = torch.empty(held, dtype=torch.uint8, device="cuda")
+        for kw in ({"tile_cfg": 9}, {"autotune": True}):
+            ddc = api.Ddc(c.V, c.J, dev(c.vox, torch.int32), dev(c.blt, torch.int32), dev(c.val, torch.float32),
+                          dtype="bf16", **kw)
+            bytes_ = api.ddc_stream_bytes(ddc.h)
+            assert bytes_ == (0, 0) if held else bytes_[1] > 0 or "autotune" in kw
+            if "tile_cfg" in kw:
+                pi = torch.empty(c.J, device="cuda")
+                api.beamlet_price(ddc.h, g, pi)
+                out.append(host(pi))
+            ddc.close()
+        del block
+        torch.cuda.empty_cache()
+    assert np.array_equal(out[0].view(np.uint32), out[1].view(np.uint32))
