@@ -107,7 +107,7 @@ struct Batch {
     int64_t device_bytes = 0;
     SpmvPlan *d_spmv = nullptr;
     int64_t *d_rows_off = nullptr, tot_rows = 0;
-    int32_t n_strm = 0; // plans whose CSR(D^T) holds a packed stream
+    int32_t n_strm = 0; // plans whose D^T g reads a packed stream
     PricePlan *d_price = nullptr;
     int64_t *d_price_off = nullptr, tot_price = 0;
     int32_t max_cols = 1;
@@ -468,21 +468,28 @@ static vmat_status make_batch(Batch &b, int32_t n_plans, const vmat_plan_desc *p
         VMAT_CUDA(cudaEventCreate(&e0));
         VMAT_CUDA(cudaEventCreate(&e1));
         float best = 1e30f;
+        const int32_t held = b.n_strm;
         for (int cfg = 0; cfg < spmv_n_configs() && cfg < 32; ++cfg) {  // warp-row families only
             if (!spmv_batched_config(cfg)) continue;
-            VMAT_TRY(spmv_rows_batched(b.dt, cfg, b.d_spmv, b.d_rows_off, n_plans, b.n_strm, b.tot_rows, s, b.cols.data(),
-                                       (int)b.cols.size())); // warm-up
-            VMAT_CUDA(cudaEventRecord(e0, s));
-            VMAT_TRY(spmv_rows_batched(b.dt, cfg, b.d_spmv, b.d_rows_off, n_plans, b.n_strm, b.tot_rows, s, b.cols.data(),
-                                       (int)b.cols.size()));
-            VMAT_CUDA(cudaEventRecord(e1, s));
-            VMAT_CUDA(cudaEventSynchronize(e1));
-            float ms = 0.f;
-            VMAT_CUDA(cudaEventElapsedTime(&ms, e0, e1));
-            b.autotune_ms[cfg] = ms;
-            if (ms < best) {
-                best = ms;
-                b.spmv_cfg = cfg;
+            // the configurations that read streams are timed from the CSR too
+            for (int32_t n_strm : {held, 0}) {
+                if (n_strm == 0 && held > 0 && !spmv_config_stream(cfg)) continue;
+                VMAT_TRY(spmv_rows_batched(b.dt, cfg, b.d_spmv, b.d_rows_off, n_plans, n_strm, b.tot_rows, s,
+                                           b.cols.data(), (int)b.cols.size())); // warm-up
+                VMAT_CUDA(cudaEventRecord(e0, s));
+                VMAT_TRY(spmv_rows_batched(b.dt, cfg, b.d_spmv, b.d_rows_off, n_plans, n_strm, b.tot_rows, s,
+                                           b.cols.data(), (int)b.cols.size()));
+                VMAT_CUDA(cudaEventRecord(e1, s));
+                VMAT_CUDA(cudaEventSynchronize(e1));
+                float ms = 0.f;
+                VMAT_CUDA(cudaEventElapsedTime(&ms, e0, e1));
+                if (b.autotune_ms[cfg] == 0.f || ms < b.autotune_ms[cfg]) b.autotune_ms[cfg] = ms;
+                if (ms < best) {
+                    best = ms;
+                    b.spmv_cfg = cfg;
+                    b.n_strm = n_strm;
+                }
+                if (held == 0) break;
             }
         }
         cudaEventDestroy(e0);

@@ -301,8 +301,8 @@ extern "C" vmat_status cg_plan(vmat_ddc hd, const vmat_mlc *mlc, const vmat_voxe
     VMAT_CUDA(cudaMemcpyAsync(cpo.data(), cpo_dev, (size_t)(K + 1) * 8, cudaMemcpyDeviceToHost, s));
     // the windowed passes' SpMV configuration (autotuned handles: timed once per MLC shape)
     int dt_cfg = h.Dt.cfg;
-    VMAT_TRY(ddc_window_config(h, mlc->n_cols, K * NR, s, &dt_cfg));
     CsrMat Dt_win = h.Dt;
+    VMAT_TRY(ddc_window_config(h, mlc->n_cols, K * NR, s, &dt_cfg, &Dt_win.read_strm));
     Dt_win.cfg = dt_cfg;
     const bool z_dt = spmv_config_index16(dt_cfg);
     if (z_dt) {

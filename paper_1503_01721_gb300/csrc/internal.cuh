@@ -108,6 +108,7 @@ struct CsrMat {
     // they read col and val): see csr_build_stream.
     unsigned char *strm = nullptr; // [strm_recs] records
     int64_t strm_recs = 0;
+    bool read_strm = true;         // false: the autotuner found col and val faster all the same
     int32_t *sptr = nullptr;       // [n_rows + 1] first record of each row
     // tiles
     int cfg = 0;                 // tile configuration index
@@ -157,6 +158,7 @@ struct Ddc {
     // shape (win_ncols, win_nseg; 0 = none yet) on a handle whose configurations were autotuned
     bool tuned = false;
     int32_t win_cfg = -1, win_ncols = 0, win_nseg = 0;
+    bool win_strm = true; // the windowed passes read the stream where win_cfg does
     // Device blocks (size, pointer) and a pinned host control block of finished cg_plan
     // calls, kept for the next call on this handle (guarded by the plan cache's mutex)
     std::vector<std::pair<size_t, void *>> plan_blocks;
@@ -243,9 +245,9 @@ vmat_status spmv_prepare_tiles(CsrMat &m, int cfg, cudaStream_t s);
 // The configuration for D^T g passes over leaf-travel windows of an MLC with n_cols columns and
 // nseg = K n_rows rows: the handle's own unless it was autotuned; then every warp-row
 // configuration (and the handle's) is timed once on a pass over the middle half of every MLC
-// row and the fastest kept for that shape.  Allocates device memory and synchronises the
-// first time for a shape: not for use while capturing.
-vmat_status ddc_window_config(Ddc &h, int32_t n_cols, int32_t nseg, cudaStream_t s, int *cfg);
+// row and the fastest kept for that shape.  *read_strm as in CsrMat.  Allocates device memory and
+// synchronises the first time for a shape: not for use while capturing.
+vmat_status ddc_window_config(Ddc &h, int32_t n_cols, int32_t nseg, cudaStream_t s, int *cfg, bool *read_strm);
 // Does configuration cfg read the 16-bit column index (and so need m.col16)?
 bool spmv_config_index16(int cfg);
 // Packed stream (csr_build_stream): every row in records of STRM_ENTRIES consecutive entries,

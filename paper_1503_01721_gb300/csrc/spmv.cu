@@ -1144,7 +1144,7 @@ vmat_status spmv_run(const Ddc &h, const CsrMat &m, const float *x, float *y, co
                      cudaStream_t s, const int32_t *skip) {
     DeviceCtx *ctx;
     VMAT_TRY(device_ctx(&ctx));
-    const bool strm = m.strm && spmv_config_stream(m.cfg);
+    const bool strm = m.strm && m.read_strm && spmv_config_stream(m.cfg);
     Launch L;
     VMAT_TRY(launch_info(h.dtype, m.cfg, strm, numbering_of(mask, m.n_rows), &L));
     if (L.row) {
@@ -1314,8 +1314,34 @@ vmat_status g_for_dt(const Ddc &h, const float *g, Scratch &ws, const float **ou
     return VMAT_OK;
 }
 
+// A pass as the autotuner times it: the least of at most `reps` repetitions after `warm` untimed ones (a
+// sum would let one late launch decide a near tie); given up when two timed ones were 1.2 times
+// the best so far.
+template <typename F> static vmat_status time_pass(F &&pass, int warm, int reps, float best_ms, cudaStream_t s,
+                                                   cudaEvent_t a, cudaEvent_t b, float *out_ms) {
+    *out_ms = 1e30f;
+    for (int rep = 0; rep < warm + reps; ++rep) {
+        cudaEventRecord(a, s);
+        VMAT_TRY(pass());
+        cudaEventRecord(b, s);
+        cudaEventSynchronize(b);
+        float ms = 0.f;
+        cudaEventElapsedTime(&ms, a, b);
+        if (rep >= warm) *out_ms = std::min(*out_ms, ms);
+        if (rep == warm + 1 && *out_ms > 1.2f * best_ms) break;
+    }
+    return VMAT_OK;
+}
+
+// The candidates in the order they are timed: those most often fastest first, since the others are
+// then given up early; the tile configurations, which allocate, last.  FROM_CSR + c: configuration c from the
+// CSR beside a packed stream.
+constexpr int FROM_CSR = 100;
+static const int kTuneOrder[] = {11, 9, 10, FROM_CSR + 11, FROM_CSR + 9, FROM_CSR + 10, 12, 13, 14, 5, 4, 7, 6, 8, 0, 1, 2, 3};
+
 vmat_status spmv_autotune(Ddc &h, cudaStream_t s) {
-    // Time every configuration on the handle's own matrices and keep the fastest.
+    // Time every configuration on the handle's own matrices and keep the fastest: the consecutive-lane
+    // ones from the packed stream and from the CSR, where the matrix holds the stream.
     for (CsrMat *m : {&h.Dt, &h.D}) {
         const bool isDt = m == &h.Dt;
         if (isDt ? !h.built_Dt : !h.built_D) continue;
@@ -1329,26 +1355,29 @@ vmat_status spmv_autotune(Ddc &h, cudaStream_t s) {
         cudaEventCreate(&a);
         cudaEventCreate(&b);
         int best = m->cfg;
-        float best_ms = 1e30f;
-        for (int cfg = 0; cfg < N_CFG; ++cfg) {
+        bool best_strm = false;
+        float best_ms = 1e30f, best_strm_ms = 1e30f;
+        for (const int c : kTuneOrder) {
+            const bool from_csr = c >= FROM_CSR;
+            const int cfg = from_csr ? c - FROM_CSR : c;
+            if (from_csr && !m->strm) continue;
             if (kCfgs[cfg].family == 3 && !m->col16) continue;
-            vmat_status st = spmv_prepare_tiles(*m, cfg, s);
-            if (st != VMAT_OK) break;
-            float ms_best = 1e30f; // the least of the repetitions: a sum lets one late launch decide a near tie
-            for (int rep = 0; rep < 6; ++rep) {
-                cudaEventRecord(a, s);
-                st = isDt ? spmv_run(h, *m, x, y, h.dtype == VMAT_FP8E4M3 ? h.scale : nullptr, all_rows(), s)
-                          : dose_forward_impl(h, x, y, false, s);
-                cudaEventRecord(b, s);
-                cudaEventSynchronize(b);
-                float ms = 0.f;
-                cudaEventElapsedTime(&ms, a, b);
-                if (rep >= 2) ms_best = std::min(ms_best, ms);
-                if (st != VMAT_OK) break;
-            }
-            if (st == VMAT_OK && ms_best < best_ms) {
-                best_ms = ms_best;
+            const bool strm = !from_csr && m->strm && spmv_config_stream(cfg);
+            if (spmv_prepare_tiles(*m, cfg, s) != VMAT_OK) break;
+            m->read_strm = strm;
+            float ms = 1e30f;
+            const vmat_status st = time_pass(
+                [&] {
+                    return isDt ? spmv_run(h, *m, x, y, h.dtype == VMAT_FP8E4M3 ? h.scale : nullptr, all_rows(), s)
+                                : dose_forward_impl(h, x, y, false, s);
+                },
+                2, 4, best_ms, s, a, b, &ms);
+            if (st != VMAT_OK) continue;
+            if (strm) best_strm_ms = std::min(best_strm_ms, ms);
+            if (ms < best_ms) {
+                best_ms = ms;
                 best = cfg;
+                best_strm = strm;
             }
         }
         cudaEventDestroy(a);
@@ -1356,8 +1385,10 @@ vmat_status spmv_autotune(Ddc &h, cudaStream_t s) {
         cudaFree(x);
         cudaFree(y);
         VMAT_TRY(spmv_prepare_tiles(*m, best, s));
-        // CSR(D) is read in this configuration only; CSR(D^T)'s windowed passes and batches choose their own
-        if (!isDt && m->strm && !spmv_config_stream(best)) {
+        m->read_strm = best_strm;
+        // A stream that lost is given back.  CSR(D) is read in this configuration only; CSR(D^T)'s windowed
+        // passes and batches choose their own, so its stream stays when it lost by less than 5%.
+        if (m->strm && !best_strm && (!isDt || best_strm_ms > 1.05f * best_ms)) {
             VMAT_CUDA(cudaStreamSynchronize(s));
             cudaFree(m->strm);
             cudaFree(m->sptr);
@@ -1367,6 +1398,7 @@ vmat_status spmv_autotune(Ddc &h, cudaStream_t s) {
         }
     }
     VMAT_CUDA(cudaStreamSynchronize(s));
+    clear_error();
     h.tuned = true;
     h.win_ncols = h.win_nseg = 0;
     return VMAT_OK;
@@ -1380,11 +1412,14 @@ __global__ void half_windows_kernel(short2 *win, int32_t nseg, int32_t n_cols) {
         win[q] = make_short2(lo, hi);
 }
 
-vmat_status ddc_window_config(Ddc &h, int32_t n_cols, int32_t nseg, cudaStream_t s, int *cfg) {
+vmat_status ddc_window_config(Ddc &h, int32_t n_cols, int32_t nseg, cudaStream_t s, int *cfg,
+                              bool *read_strm) {
     *cfg = h.Dt.cfg;
+    *read_strm = h.Dt.read_strm;
     if (!h.tuned || h.Dt.nnz == 0) return VMAT_OK;
     if (h.win_ncols == n_cols && h.win_nseg == nseg) {
         *cfg = h.win_cfg;
+        *read_strm = h.win_strm;
         return VMAT_OK;
     }
     DevBuf bw, bo, bx, by;
@@ -1403,27 +1438,28 @@ vmat_status ddc_window_config(Ddc &h, int32_t n_cols, int32_t nseg, cudaStream_t
     VMAT_CUDA(cudaEventCreate(&a));
     VMAT_CUDA(cudaEventCreate(&b));
     int best = h.Dt.cfg;
+    bool best_strm = h.Dt.read_strm;
     float best_ms = 1e30f;
-    for (int c = 0; c < N_CFG; ++c) {
-        const int fam = kCfgs[c].family;
-        if (c != h.Dt.cfg && !(fam == 1 || fam == 2 || (fam == 3 && h.Dt.col16))) continue;
+    // (from the CSR beside a stream only where the CSR won a pass over every row)
+    for (const int c : kTuneOrder) {
+        const bool from_csr = c >= FROM_CSR;
+        const int k = from_csr ? c - FROM_CSR : c, fam = kCfgs[k].family;
+        if (from_csr && (!h.Dt.strm || h.Dt.read_strm)) continue;
+        if (k != h.Dt.cfg && !(fam == 1 || fam == 2 || (fam == 3 && h.Dt.col16))) continue;
         CsrMat m = h.Dt;
-        m.cfg = c; // a warp-row configuration reads no tile structure; the handle's own has its tiles
-        float tot = 1e30f; // the least of the repetitions
-        vmat_status st = VMAT_OK;
-        for (int rep = 0; rep < 4 && st == VMAT_OK; ++rep) {
-            cudaEventRecord(a, s);
-            st = spmv_run(h, m, static_cast<const float *>(bx.p), static_cast<float *>(by.p),
-                          h.dtype == VMAT_FP8E4M3 ? h.scale : nullptr, mask, s);
-            cudaEventRecord(b, s);
-            cudaEventSynchronize(b);
-            float ms = 0.f;
-            cudaEventElapsedTime(&ms, a, b);
-            if (rep >= 1) tot = std::min(tot, ms);
-        }
-        if (st == VMAT_OK && tot < best_ms) {
-            best_ms = tot;
-            best = c;
+        m.cfg = k; // a warp-row configuration reads no tile structure; the handle's own has its tiles
+        m.read_strm = !from_csr;
+        float ms = 1e30f;
+        const vmat_status st = time_pass(
+            [&] {
+                return spmv_run(h, m, static_cast<const float *>(bx.p), static_cast<float *>(by.p),
+                                h.dtype == VMAT_FP8E4M3 ? h.scale : nullptr, mask, s);
+            },
+            1, 3, best_ms, s, a, b, &ms);
+        if (st == VMAT_OK && ms < best_ms) {
+            best_ms = ms;
+            best = k;
+            best_strm = m.read_strm;
         }
     }
     cudaEventDestroy(a);
@@ -1431,9 +1467,11 @@ vmat_status ddc_window_config(Ddc &h, int32_t n_cols, int32_t nseg, cudaStream_t
     VMAT_CUDA(cudaStreamSynchronize(s));
     clear_error();
     h.win_cfg = best;
+    h.win_strm = best_strm;
     h.win_ncols = n_cols;
     h.win_nseg = nseg;
     *cfg = best;
+    *read_strm = best_strm;
     return VMAT_OK;
 }
 
