@@ -219,7 +219,8 @@ vmat_status ddc_load_coo(int32_t V, int32_t J, int64_t nnz, const int32_t *vox, 
  * Index checks and the duplicate check report VMAT_EINVAL.  Synchronises. */
 vmat_status ddc_build(vmat_ddc h, const vmat_build_opts *opts, void *stream);
 
-/* Release every device buffer of the handle.  NULL is accepted. */
+/* Release every device buffer of the handle, and the device memory that the library keeps between
+ * calls (see mp_bb_solve).  NULL is accepted. */
 vmat_status ddc_free(vmat_ddc h);
 
 /* Sizes and build facts of a handle (host struct). */
@@ -345,8 +346,8 @@ vmat_status aperture_grad(const vmat_mlc *mlc, int32_t n_ap, const int32_t *cps,
  * solution out.  z: device float [V], receives DA y.  opts NULL = defaults
  * (500, 1e-6, 1e-9, 1e-12, 1e12).  rep: HOST struct or NULL.
  * The step lengths, objective and stopping tests use FP64; the products FP32.
- * Synchronises.  Scratch of up to 128 MB stays with the calling thread for its next
- * call (freed when the thread ends); more comes from the stream-ordered pool. */
+ * Synchronises.  Its scratch comes from a stream-ordered pool of the library's own, which keeps up
+ * to 128 MB per device between calls (ddc_free gives it back). */
 vmat_status mp_bb_solve(const float *DA, int32_t V, int32_t n_ap, int64_t ld, const vmat_voxels *vox,
                         const float *lo, const float *hi, float *y, float *z, const vmat_bb_opts *opts,
                         vmat_bb_report *rep, void *stream);

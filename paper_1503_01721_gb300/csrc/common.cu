@@ -42,6 +42,18 @@ vmat_status device_ctx(DeviceCtx **out) {
         VMAT_CUDA(cudaMalloc(&c->status, sizeof(int32_t)));
         VMAT_CUDA(cudaMemset(c->status, 0, sizeof(int32_t)));
         VMAT_CUDA(cudaDeviceSynchronize());
+        cudaMemPoolProps props = {};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.handleTypes = cudaMemHandleTypeNone;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        uint64_t keep = KEPT_BYTES;
+        if (cudaMemPoolCreate(&c->kept, &props) != cudaSuccess ||
+            cudaMemPoolSetAttribute(c->kept, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+            if (c->kept) cudaMemPoolDestroy(c->kept);
+            c->kept = nullptr;
+            cudaGetLastError();
+        }
         g_ctx[dev] = c;
     }
     *out = g_ctx[dev];
@@ -52,6 +64,15 @@ vmat_status Scratch::alloc(size_t bytes, cudaStream_t s) {
     stream = s;
     if (bytes == 0) bytes = 16;
     VMAT_CUDA(cudaMallocAsync(&ptr, bytes, s));
+    return VMAT_OK;
+}
+
+vmat_status Scratch::alloc_kept(size_t bytes, cudaStream_t s) {
+    DeviceCtx *ctx;
+    VMAT_TRY(device_ctx(&ctx));
+    if (!ctx->kept) return alloc(bytes, s);
+    stream = s;
+    VMAT_CUDA(cudaMallocFromPoolAsync(&ptr, bytes ? bytes : 16, ctx->kept, s));
     return VMAT_OK;
 }
 
@@ -325,6 +346,8 @@ vmat_status ddc_free(vmat_ddc hd) {
     cudaDeviceSynchronize();
     h->free_all();
     delete h;
+    DeviceCtx *ctx;
+    if (device_ctx(&ctx) == VMAT_OK && ctx->kept) cudaMemPoolTrimTo(ctx->kept, 0); // what is not in use
     return VMAT_OK;
 }
 

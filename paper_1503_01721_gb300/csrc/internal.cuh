@@ -53,7 +53,13 @@ struct DeviceCtx {
     int device = -1;
     int n_sm = 0;
     int32_t *status = nullptr; // device int32, OR-ed by kernels
+    // The library's own stream-ordered pool (null where the device has none), for scratch of calls that
+    // synchronise: the default pool gives everything back at each synchronisation, and mapping
+    // it again took longer than a small call.  It keeps at most KEPT_BYTES, for all threads and streams together
+    // (a block freed on one stream is reused on another only behind it), and ddc_free empties it.
+    cudaMemPool_t kept = nullptr;
 };
+constexpr size_t KEPT_BYTES = (size_t)128 << 20;
 vmat_status device_ctx(DeviceCtx **out);
 
 inline cudaStream_t as_stream(void *s) { return reinterpret_cast<cudaStream_t>(s); }
@@ -66,6 +72,7 @@ struct Scratch {
         if (ptr) cudaFreeAsync(ptr, stream);
     }
     vmat_status alloc(size_t bytes, cudaStream_t s);
+    vmat_status alloc_kept(size_t bytes, cudaStream_t s); // from DeviceCtx::kept
 };
 
 // Device buffer freed at scope exit unless released (build and set-up steps).

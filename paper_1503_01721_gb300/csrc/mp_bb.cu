@@ -2126,40 +2126,6 @@ vmat_status mp_bb_enqueue_batched(const void *args, const int64_t *weight, unsig
     return VMAT_OK;
 }
 
-// Scratch of mp_bb_impl that a thread keeps between calls: the call returns only after its
-// stream has been synchronised, so the next call of the thread may use it on any stream.
-// At most MP_KEEP_BYTES; freed when the thread ends, or when a larger one or another device is
-// needed.  (From the stream-ordered pool, which gives its memory back at each synchronisation,
-// the 70 MB of a 422K-voxel, 40-aperture problem were mapped anew in every call.)
-constexpr size_t MP_KEEP_BYTES = (size_t)128 << 20;
-struct MpKeep {
-    void *p = nullptr;
-    size_t bytes = 0;
-    int dev = -1;
-    void drop() {
-        if (p) cudaFree(p);
-        p = nullptr;
-        bytes = 0;
-        dev = -1;
-    }
-    ~MpKeep() { drop(); }
-};
-static void *mp_keep(size_t bytes, int dev) {
-    static thread_local MpKeep k;
-    if (bytes > MP_KEEP_BYTES) return nullptr;
-    if (k.dev != dev || k.bytes < bytes) {
-        k.drop();
-        if (cudaMalloc(&k.p, bytes) != cudaSuccess) {
-            cudaGetLastError();
-            k.p = nullptr;
-            return nullptr;
-        }
-        k.bytes = bytes;
-        k.dev = dev;
-    }
-    return k.p;
-}
-
 vmat_status mp_bb_impl(const float *DA, int32_t V, int32_t n_ap, int64_t ld, const uint8_t *struct_id,
                        int64_t wstride, const vmat_voxels *vox, const float *lo, const float *hi, float *y,
                        float *z, const vmat_bb_opts *opts_in, double F_offset, vmat_bb_report *rep, cudaStream_t s) {
@@ -2177,12 +2143,11 @@ vmat_status mp_bb_impl(const float *DA, int32_t V, int32_t n_ap, int64_t ld, con
     const size_t conv_bytes =
         wstride == 0 ? (((size_t)n_wtiles * mp_wtile_stride(n_ap) * sizeof(float) + 255) & ~(size_t)255) : 0;
     const size_t bytes = conv_bytes + mp_ws_bytes(n_ap, p_max);
-    Scratch own; // when the thread's kept scratch does not hold it
-    void *mem = mp_keep(bytes, ctx->device);
-    if (!mem) {
-        VMAT_TRY(own.alloc(bytes, s));
-        mem = own.ptr;
-    }
+    // (from the default pool the 70 MB of a 422K-voxel, 40-aperture problem were mapped anew in every
+    // call: 3.8 ms for a new state's first pass instead of 2.7)
+    Scratch own;
+    VMAT_TRY(own.alloc_kept(bytes, s));
+    void *const mem = own.ptr;
     void *const ws = static_cast<char *>(mem) + conv_bytes;
     // a column-major input is copied once into the warp-tile layout (with the labels)
     if (wstride == 0) {
