@@ -10,7 +10,9 @@ D x and D^T g pass the plan makes, divided by the plan's wall time (GB/s).
 The D^T g passes read only the beamlet rows inside the leaf-travel windows of
 the unoccupied CPs (the prices that pricing reads), so their bytes are those
 rows' bytes; plan.pp1_window_frac = those bytes over the bytes of passes over
-every row of the unoccupied CPs.  ms_per_step = plan wall time.  roofline =
+every row of the unoccupied CPs.  ms_per_step = plan wall time.  Passes that read
+the matrix's packed stream are counted at the CSR's bytes in value (an effective
+rate); roofline and the fractions use the bytes they move.  roofline =
 the beamlet-price SpMV, timed by the library's CUDA events on its launch
 stream during the timed plans.
 
@@ -49,18 +51,21 @@ WORKLOAD_DESC = DESCS[WORKLOAD]
 SPMV_KERNELS = {0: "spmv_tile_kernel<256,16,2>", 1: "spmv_tile_kernel<256,8,3>", 2: "spmv_tile_kernel<512,8,2>",
                 3: "spmv_tile_kernel<128,16,3>", 4: "spmv_warp_row_kernel<256,2>", 5: "spmv_warp_row_kernel<256,1>",
                 6: "spmv_warp_row_kernel<512,4>", 7: "spmv_warp_row_kernel<256,4>", 8: "spmv_warp_row_kernel<256,8>",
-                # 9-11 read the packed stream of the matrix (spmv_warp_row_c_kernel where there is none)
-                9: "spmv_warp_row_x_kernel<256,8>", 10: "spmv_warp_row_x_kernel<256,6>",
-                11: "spmv_warp_row_x_kernel<512,4>", 12: "spmv_warp_row_z_kernel<256,4>",
+                9: "spmv_warp_row_c_kernel<256,4>", 10: "spmv_warp_row_c_kernel<256,8>",
+                11: "spmv_warp_row_c_kernel<512,4>", 12: "spmv_warp_row_z_kernel<256,4>",
                 13: "spmv_warp_row_z_kernel<256,8>", 14: "spmv_warp_row_z_kernel<512,4>"}
+# the same where the pass reads the packed stream of the matrix (api.ddc_stream_reads)
+STREAM_KERNELS = {9: "spmv_warp_row_x_kernel<256,8>", 10: "spmv_warp_row_x_kernel<256,6>",
+                  11: "spmv_warp_row_x_kernel<512,4>"}
 # configurations that read the 16-bit column index (built with index16)
 INDEX16_CFGS = (12, 13, 14)
-# DRAM traffic over algorithmic bytes of the plan's windowed D^T g launches, per (value type,
-# configuration, CSR(D^T) column order): dram__bytes_read.sum + dram__bytes_write.sum over the 30
-# windowed launches of the 45-CP plan (the same kernels on a quarter of the CPs), over their algorithmic
-# bytes, from one ncu capture each; a configuration without such a capture reports null
-# (9 and 10 since they read the packed stream, which moves less than the CSR's bytes).
-WINDOWED_TRAFFIC_RATIO = {("f32", 5, "voxel"): 0.9988, ("f32", 11, "brick"): 0.8407}
+# DRAM traffic over the CSR's bytes of the plan's windowed D^T g launches, per (value type,
+# configuration, CSR(D^T) column order, what it reads): dram__bytes_read.sum + dram__bytes_write.sum over the 30
+# windowed launches of the 45-CP plan (the same kernels on a quarter of the CPs), over their CSR
+# bytes, from one ncu capture each; a configuration without such a capture reports null.
+WINDOWED_TRAFFIC_RATIO = {("f32", 5, "voxel", "csr"): 0.9988, ("f32", 9, "voxel", "csr"): 1.0010,
+                          ("f32", 11, "voxel", "csr"): 1.0009, ("f32", 9, "brick", "csr"): 1.0039,
+                          ("f32", 11, "brick", "csr"): 1.0038, ("f32", 11, "brick", "stream"): 0.8244}
 # The paper's own plan times (Table 2 and Table 3): other hardware, patient data and aperture
 # counts, so context for the line, not a baseline of its metric.
 PAPER_CONTEXT = {
@@ -534,21 +539,32 @@ def run_ours(args, rank, world, local):
     spmv_n = sum(s["pp1_spmv_launches"] for s in stats_all)
     spmv_bytes = sum(s["pp1_spmv_bytes"] for s in stats_all)
     peaks = roofline.measured_peaks()
-    achieved = spmv_bytes / (spmv_ms * 1e-3) / 1e9
     cfg_dt = int(stats_all[-1]["pp1_spmv_cfg"])  # the windowed passes' configuration
-    kname = SPMV_KERNELS.get(cfg_dt, f"spmv configuration {cfg_dt}") + \
+    # bytes moved: a stream's records, in the proportion to the CSR's bytes that the whole matrix has
+    strm, reads = api.ddc_stream_bytes(h), api.ddc_stream_reads(h)
+    n_sc = case.J if args.dtype == "fp8" else 0
+    b_dt = roofline.spmv_bytes(case.nnz, case.J, case.V, case.J, args.dtype, n_sc)
+    b_d = roofline.spmv_bytes(case.nnz, info["n_active_vox"], case.J, case.V, args.dtype, n_sc)
+    m_dt = roofline.stream_bytes(strm[1], case.J, case.V, case.J, n_sc)
+    moved_dt = m_dt if reads["Dt"] else b_dt
+    moved_d = roofline.stream_bytes(strm[0], info["n_active_vox"], case.J, case.V, n_sc) if reads["D"] else b_d
+    moved_ratio = m_dt / b_dt if reads["windows"] else 1.0
+    achieved = spmv_bytes * moved_ratio / (spmv_ms * 1e-3) / 1e9
+    kname = (STREAM_KERNELS if reads["windows"] else SPMV_KERNELS).get(cfg_dt, f"spmv configuration {cfg_dt}") + \
         (" + spmv_fixup" if cfg_dt < 4 else "") + " (beamlet price D^T g over the unoccupied CPs)"
     bytes_launch = spmv_bytes / max(spmv_n, 1)
-    ratio = WINDOWED_TRAFFIC_RATIO.get((args.dtype, cfg_dt, "brick" if info["vox_brick"] else "voxel"))
+    ratio = WINDOWED_TRAFFIC_RATIO.get((args.dtype, cfg_dt, "brick" if info["vox_brick"] else "voxel",
+                                        "stream" if reads["windows"] else "csr"))
     roof = {"bound": "hbm", "kernel": kname,
             "achieved": round(achieved, 1), "peak": peaks["hbm_gbs"], "unit": "GB/s",
             "frac": round(achieved / peaks["hbm_gbs"], 4),
             "traffic": None if ratio is None else round(ratio * bytes_launch),
             "traffic_source": None if ratio is None else
-            f"ncu dram bytes / algorithmic bytes = {ratio} for this kernel over the windowed D^T g launches of "
-            "the 45-CP plan, times this launch's algorithmic bytes",
+            f"ncu dram bytes / the CSR's bytes = {ratio} for this kernel over the windowed D^T g launches of "
+            "the 45-CP plan, times this launch's CSR bytes",
             "peak_source": peaks["source"], "frac_of_nominal": round(achieved / roofline.HBM_NOMINAL_GBS, 4),
-            "nominal_peak": roofline.HBM_NOMINAL_GBS, "bytes_per_launch": round(bytes_launch),
+            "nominal_peak": roofline.HBM_NOMINAL_GBS, "bytes_per_launch": round(bytes_launch * moved_ratio),
+            "csr_bytes_per_launch": round(bytes_launch), "reads_stream": reads["windows"],
             "avg_launch_ms": round(spmv_ms / max(spmv_n, 1), 4)}
 
     # the last timed plan's final dose against float64 sums over the COO at sampled voxels
@@ -586,14 +602,14 @@ def run_ours(args, rank, world, local):
 
     t_dt = median_ms(lambda: api.beamlet_price(h, g, pi))
     t_d = median_ms(lambda: api.dose_forward(h, x, d))
-    b_dt = roofline.spmv_bytes(case.nnz, case.J, case.V, case.J, args.dtype, case.J if args.dtype == "fp8" else 0)
-    b_d = roofline.spmv_bytes(case.nnz, info["n_active_vox"], case.J, case.V, args.dtype,
-                              case.J if args.dtype == "fp8" else 0)
+    # *_gbs: effective, the CSR's bytes; the fractions: the bytes moved
     pair = {"timing": f"median of {reps} passes each", "dt_g_ms": round(t_dt, 4),
             "dt_g_gbs": round(b_dt / t_dt / 1e6, 1), "d_x_ms": round(t_d, 4),
             "d_x_gbs": round(b_d / t_d / 1e6, 1), "pair_gbs": round((b_dt + b_d) / (t_dt + t_d) / 1e6, 1),
-            "pair_frac": round((b_dt + b_d) / (t_dt + t_d) / 1e6 / peaks["hbm_gbs"], 4),
-            "pair_frac_of_nominal": round((b_dt + b_d) / (t_dt + t_d) / 1e6 / roofline.HBM_NOMINAL_GBS, 4)}
+            "reads_stream": {"dt_g": reads["Dt"], "d_x": reads["D"]},
+            "dt_g_moved_gbs": round(moved_dt / t_dt / 1e6, 1), "d_x_moved_gbs": round(moved_d / t_d / 1e6, 1),
+            "pair_frac": round((moved_dt + moved_d) / (t_dt + t_d) / 1e6 / peaks["hbm_gbs"], 4),
+            "pair_frac_of_nominal": round((moved_dt + moved_d) / (t_dt + t_d) / 1e6 / roofline.HBM_NOMINAL_GBS, 4)}
 
     # end to end through the C ABI with host buffers: H2D of the COO, build, plan, D2H of the results
     dose_h = torch.empty(case.V, dtype=torch.float32).pin_memory()
@@ -860,7 +876,8 @@ def batch_measure(workload, dtype, steps, warmup):
     peaks = roofline.measured_peaks()
     out = {"mode": "batch", "workload": workload, "n_plans": len(specs), "nnz": nnz, "dtype": dtype,
            "batched": {"ms_per_run": round(ms_batch, 3), "gbs": round(bytes_run / ms_batch / 1e6, 1),
-                       "frac_of_hbm": round(bytes_run / ms_batch / 1e6 / peaks["hbm_gbs"], 4)},
+                       # effective bytes (the CSR's) over the copy bandwidth: not a fraction of what moved
+                       "effective_over_hbm": round(bytes_run / ms_batch / 1e6 / peaks["hbm_gbs"], 4)},
            "one_by_one": {"ms_per_run": round(ms_seq, 3), "gbs": round(bytes_seq / ms_seq / 1e6, 1)},
            "speedup": round(ms_seq / ms_batch, 3), "bb_iters": sum(s["bb_iters_total"] for s in stb),
            "apertures": [s["n_apertures"] for s in stb], "F_rel_diff_max": max(rel),

@@ -179,7 +179,8 @@ typedef struct {
     double t_final_ms;  /* final dose D (A y) and objective */
     double pp1_spmv_ms; /* the D^T g kernels alone */
     int64_t pp1_spmv_launches;
-    double pp1_spmv_bytes;  /* algorithmic bytes of those launches (rows inside the leaf-travel windows) */
+    double pp1_spmv_bytes;  /* algorithmic bytes of those launches (rows inside the leaf-travel windows), in
+                               the CSR's format also where the packed stream is read, which moves fewer */
     double other_spmv_bytes; /* algorithmic bytes of the D x / aperture-dose passes */
     int32_t n_apertures;
     int32_t bb_iters_total;
@@ -227,8 +228,12 @@ vmat_status ddc_free(vmat_ddc h);
 vmat_status ddc_info(vmat_ddc h, vmat_ddc_info *out);
 
 /* Device bytes of each CSR's packed stream (build option autotune, configurations 9-11), 0 where
- * the handle holds none.  They come on top of vmat_ddc_info's bytes_D and bytes_Dt. */
-vmat_status vmat_ddc_stream_bytes(vmat_ddc h, int64_t *bytes_D, int64_t *bytes_Dt);
+ * the handle holds none.  They come on top of vmat_ddc_info's bytes_D and bytes_Dt.  *reads: which
+ * passes read their stream (VMAT_STREAM_*; the windowed D^T g of the last MLC shape planned for). */
+#define VMAT_STREAM_D 1
+#define VMAT_STREAM_DT 2
+#define VMAT_STREAM_WINDOWS 4
+vmat_status vmat_ddc_stream_bytes(vmat_ddc h, int64_t *bytes_D, int64_t *bytes_Dt, int32_t *reads);
 
 /* ---- Sparse products (hot path) ------------------------------------------ */
 

@@ -80,7 +80,7 @@ SIGNATURES = {
     "ddc_build": (c_i32, [c_vp, ctypes.POINTER(BuildOpts), c_vp]),
     "ddc_free": (c_i32, [c_vp]),
     "ddc_info": (c_i32, [c_vp, ctypes.POINTER(DdcInfo)]),
-    "vmat_ddc_stream_bytes": (c_i32, [c_vp, ctypes.POINTER(c_i64), ctypes.POINTER(c_i64)]),
+    "vmat_ddc_stream_bytes": (c_i32, [c_vp, ctypes.POINTER(c_i64), ctypes.POINTER(c_i64), ctypes.POINTER(c_i32)]),
     "dose_forward": (c_i32, [c_vp, c_vp, c_vp, c_vp]),
     "beamlet_price": (c_i32, [c_vp, c_vp, c_vp, c_vp, c_i32, c_vp]),
     "beamlet_price_windowed": (c_i32, [c_vp, c_vp, c_vp, c_vp, c_vp, c_vp, c_vp]),

@@ -136,11 +136,22 @@ def ddc_info(h: int) -> dict:
     return {f: getattr(info, f) for f, _ in info._fields_}
 
 
+def _stream_facts(h: int):
+    d, dt, reads = ctypes.c_int64(), ctypes.c_int64(), ctypes.c_int32()
+    check("vmat_ddc_stream_bytes", _lib.load().vmat_ddc_stream_bytes(ctypes.c_void_p(h), ctypes.byref(d),
+                                                                     ctypes.byref(dt), ctypes.byref(reads)))
+    return d.value, dt.value, reads.value
+
+
 def ddc_stream_bytes(h: int) -> tuple:
     """Device bytes of the packed streams of CSR(D) and CSR(D^T), 0 where the handle holds none."""
-    d, dt = ctypes.c_int64(), ctypes.c_int64()
-    check("vmat_ddc_stream_bytes", _lib.load().vmat_ddc_stream_bytes(ctypes.c_void_p(h), ctypes.byref(d), ctypes.byref(dt)))
-    return d.value, dt.value
+    return _stream_facts(h)[:2]
+
+
+def ddc_stream_reads(h: int) -> dict:
+    """Which passes read a packed stream: D x, D^T g, and the windowed D^T g of the last MLC shape planned for."""
+    r = _stream_facts(h)[2]
+    return {"D": bool(r & 1), "Dt": bool(r & 2), "windows": bool(r & 4)}
 
 
 # ---------------------------------------------------------------------------- products

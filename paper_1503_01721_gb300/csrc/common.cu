@@ -382,9 +382,9 @@ vmat_status ddc_info(vmat_ddc hd, vmat_ddc_info *out) {
     return VMAT_OK;
 }
 
-vmat_status vmat_ddc_stream_bytes(vmat_ddc hd, int64_t *bytes_D, int64_t *bytes_Dt) {
+vmat_status vmat_ddc_stream_bytes(vmat_ddc hd, int64_t *bytes_D, int64_t *bytes_Dt, int32_t *reads) {
     clear_error();
-    if (!hd || !bytes_D || !bytes_Dt) return set_error(VMAT_EINVAL, "vmat_ddc_stream_bytes: NULL argument");
+    if (!hd || !bytes_D || !bytes_Dt || !reads) return set_error(VMAT_EINVAL, "vmat_ddc_stream_bytes: NULL argument");
     const Ddc *h = as_ddc(hd);
     const int vb = value_bytes(h->dtype);
     auto bytes = [&](const CsrMat &m) {
@@ -392,6 +392,11 @@ vmat_status vmat_ddc_stream_bytes(vmat_ddc hd, int64_t *bytes_D, int64_t *bytes_
     };
     *bytes_D = bytes(h->D);
     *bytes_Dt = bytes(h->Dt);
+    auto reads_it = [](const CsrMat &m, int cfg, bool read_strm) { return m.strm && read_strm && spmv_config_stream(cfg); };
+    const bool win = h->win_nseg > 0; // a windowed configuration was timed; else it is CSR(D^T)'s
+    *reads = (reads_it(h->D, h->D.cfg, h->D.read_strm) ? VMAT_STREAM_D : 0) |
+             (reads_it(h->Dt, h->Dt.cfg, h->Dt.read_strm) ? VMAT_STREAM_DT : 0) |
+             (reads_it(h->Dt, win ? h->win_cfg : h->Dt.cfg, win ? h->win_strm : h->Dt.read_strm) ? VMAT_STREAM_WINDOWS : 0);
     return VMAT_OK;
 }
 

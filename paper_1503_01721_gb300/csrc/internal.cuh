@@ -281,12 +281,12 @@ int32_t spmv_config_tile(int cfg);
 vmat_status dose_forward_impl(const Ddc &h, const float *x, float *d, bool compact, cudaStream_t s);
 
 // Algorithmic bytes of the matrix part of one SpMV pass over `rows` rows holding
-// `nnz` nonzeros and `chunks` 16-bit-index chunks, in the format configuration
-// cfg reads: each value (vb bytes) and column index (4, or 2 plus a 4-byte base
-// per chunk and an 8-byte chunk pointer per row) once, an 8-byte row pointer
-// per row.  Dense inputs, outputs and scales are the caller's.  Where configurations 9-11 read
-// the packed stream these stay the CSR's bytes (the metric's definition); the stream moves
-// about 0.83 (FP32), 0.78 (BF16) and 0.72 (FP8) of them at 1,300 entries per row.
+// `nnz` nonzeros and `chunks` 16-bit-index chunks: each value (vb bytes) and column index (4, or for the
+// configurations that read the 16-bit index 2 plus a 4-byte base per chunk and an 8-byte chunk
+// pointer per row) once, an 8-byte row pointer per row.  Dense inputs, outputs and scales are the
+// caller's.  A pass that reads the packed stream is counted at the CSR's bytes too, the metric's
+// definition (an effective rate, not one to hold against a peak); the stream moves about 0.83 (FP32),
+// 0.78 (BF16) and 0.72 (FP8) of them at 1,300 entries per row (vmat_ddc_stream_bytes).
 inline double csr_pass_bytes(int cfg, int vb, double nnz, double rows, double chunks) {
     if (spmv_config_index16(cfg)) return nnz * (vb + 2) + 4.0 * chunks + 16.0 * rows;
     return nnz * (vb + 4) + 8.0 * rows;

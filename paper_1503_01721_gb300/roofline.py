@@ -40,6 +40,12 @@ def spmv_bytes_index16(nnz: int, n_chunks: int, n_rows: int, n_in: int, n_out: i
             + 4 * n_in + 4 * n_out + 4 * n_scales)
 
 
+def stream_bytes(strm_bytes: int, n_rows: int, n_in: int, n_out: int, n_scales: int = 0) -> int:
+    """Bytes y = M x moves reading the packed stream: strm_bytes (the padded records and their 4-byte
+    row pointers, api.ddc_stream_bytes) and what the CSR pass moves beside its entries."""
+    return strm_bytes + PTR_BYTES * (n_rows + 1) + 4 * n_in + 4 * n_out + 4 * n_scales
+
+
 def measured_peaks(path: str | None = None) -> dict:
     """Peaks measured on this GPU model (copy bandwidth, bf16 GEMM), if recorded."""
     if path is None:

@@ -188,3 +188,15 @@ def test_the_stream_gives_way_when_memory_is_short():
         del block
         torch.cuda.empty_cache()
     assert np.array_equal(out[0].view(np.uint32), out[1].view(np.uint32))
+
+
+def test_which_passes_read_a_stream():
+    from paper_1503_01721_gb300 import api
+    c = synth.make_case("cfg1", seed=0)
+
+    def reads(**kw):
+        ddc = make_ddc(c, "bf16", **kw)
+        return api.ddc_stream_reads(ddc.h)
+    assert reads(tile_cfg=9) == {"D": True, "Dt": True, "windows": True}
+    assert reads(tile_cfg=4) == {"D": False, "Dt": False, "windows": False}
+    assert reads(tile_cfg=12, index16=True) == {"D": False, "Dt": False, "windows": False}
