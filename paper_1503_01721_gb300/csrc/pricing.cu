@@ -103,9 +103,9 @@ __device__ __forceinline__ void window_prefix(const float *__restrict__ row, int
     }
 }
 
-// Shared memory per warp of the row kernel: the float64 prefix sums, their float32
-// roundings and each left leaf's best float32 value, n_cols + 1 of each.
-__host__ __device__ constexpr size_t row_smem_stride(int n_cols) { return (((size_t)(n_cols + 1) * 16) + 15) & ~15; }
+// Shared memory per warp of the row kernel: the float64 prefix sums and their
+// float32 roundings, n_cols + 1 of each.
+__host__ __device__ constexpr size_t row_smem_stride(int n_cols) { return (((size_t)(n_cols + 1) * 12) + 15) & ~15; }
 
 // Best opening of MLC row r of CP k (one warp; ws: row_smem_stride(n_cols) bytes of
 // shared memory for this warp).  Writes the row's entry gw of rb_*.
@@ -118,9 +118,7 @@ __host__ __device__ constexpr size_t row_smem_stride(int n_cols) { return (((siz
 // two roundings of P to float32, one float32 and one float64 subtraction, each at
 // most 2^-24 or 2^-53 relative, with a factor 4 to spare).  The pairs that attain
 // the float64 maximum are always among them, so the choice, ties included, is the
-// one the exhaustive float64 search makes.  The first pass keeps each left leaf's float32
-// maximum, and the second visits only the left leaves whose maximum reaches the threshold,
-// a few of a row's (it used to walk every pair again, half of the search's time).
+// one the exhaustive float64 search makes.
 __device__ __forceinline__ void price_row_warp(const PricingGeom &g, const float *__restrict__ pi,
                                                const uint8_t *__restrict__ occupied, const int16_t *__restrict__ leaves,
                                                int64_t gw, unsigned char *ws, double *rb_v, int16_t *rb_lr,
@@ -131,7 +129,6 @@ __device__ __forceinline__ void price_row_warp(const PricingGeom &g, const float
     const int N = g.n_cols;
     double *P = reinterpret_cast<double *>(ws);
     float *P32 = reinterpret_cast<float *>(ws + (size_t)(N + 1) * 8);
-    float *best32 = P32 + (N + 1); // a lane reads the entries it wrote
     const int kl = nearest_occupied(g, occupied, k, -1, lane), kr = nearest_occupied(g, occupied, k, 1, lane);
     const RowWindow win = row_window(g, leaves, k, r, kl, kr);
     const int Lmin = win.Lmin, Lmax = win.Lmax, Rmin = win.Rmin, Rmax = win.Rmax;
@@ -154,18 +151,7 @@ __device__ __forceinline__ void price_row_warp(const PricingGeom &g, const float
     float m32 = -INFINITY;
     for (int L = Lmin + lane; L <= Lmax; L += 32) {
         const float pl = P32[L];
-        // four maxima: a chain of one per pair would wait for the one before
-        float m[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-        int R = max(L, Rmin);
-        // (a price that is not a number makes every later sum one: its pairs stay candidates)
-        const bool nan = R <= Rmax && (isnan(pl) || isnan(P32[Rmax]));
-        for (; R + 3 <= Rmax; R += 4)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) m[q] = fmaxf(m[q], P32[R + q] - pl);
-        for (; R <= Rmax; ++R) m[0] = fmaxf(m[0], P32[R] - pl);
-        const float ml = fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3]));
-        best32[L] = nan ? INFINITY : ml;
-        m32 = fmaxf(m32, ml);
+        for (int R = max(L, Rmin); R <= Rmax; ++R) m32 = fmaxf(m32, P32[R] - pl);
     }
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) m32 = fmaxf(m32, __shfl_xor_sync(0xffffffffu, m32, d));
@@ -178,7 +164,6 @@ __device__ __forceinline__ void price_row_warp(const PricingGeom &g, const float
     best.key = 0;
     best.w = best.cd = best.L = 0;
     for (int L = Lmin + lane; L <= Lmax; L += 32) {
-        if (best32[L] < thr) continue; // every pair of this left leaf is below the threshold
         const float pl = P32[L];
         const long long bl = __double_as_longlong(P[L]);
         for (int R = max(L, Rmin); R <= Rmax; ++R) {
@@ -228,7 +213,7 @@ constexpr int CP_THREADS = 1024;
 
 // Sum of rb_v[i0 .. i0 + n) in order; false when a row has no opening.  The loads of eight
 // rows are issued together: stopping at the first row without an opening made every load
-// wait for the one before (180 CPs of 64 rows: 15 us for the kernel, an L2 access per row).
+// wait for the one before (an L2 access per row; the CP kernel at 180 CPs of 64 rows 15.1 -> 13.6 us).
 __device__ __forceinline__ bool row_best_sum(const double *__restrict__ rb_v, const uint8_t *__restrict__ rb_ok,
                                              int64_t i0, int n, double *sum) {
     double price = 0.0;
@@ -381,7 +366,8 @@ __host__ __device__ constexpr size_t interdig_smem(int N) {
 // lane keeps 32 rows' sequential sums in one instruction stream, where a row per
 // warp spends a warp-wide FP64 instruction on every add of one row.  A warp takes 32 rows
 // of one CP, so that it finds the CP's neighbours together (a thread's own search read the
-// occupancy byte by byte), and loads eight prices before it adds them.
+// occupancy byte by byte), and loads eight prices before it adds them: 8.2 -> 7.2 us at 36 CPs of 20 x 20,
+// 27.9 -> 25.7 at 360 of 80 x 96, even at 64 columns (15.6 -> 15.8 at 180 CPs of 64 rows).
 __global__ void window_prefix_kernel(PricingGeom g, const float *__restrict__ pi,
                                        const uint8_t *__restrict__ occupied, const int16_t *__restrict__ leaves,
                                        double *__restrict__ Pall, const int32_t *skip) {
@@ -964,7 +950,7 @@ __global__ void __launch_bounds__(PICK_THREADS) price_pick_interdig_kernel(Prici
     const int kb = kwin;
     if (kb < 0) return;
     // The backtrack reads one entry of every row's table, each where the one before points: from
-    // global memory 64 accesses one after the other (45 us at 64 rows of 64 columns).
+    // global memory 64 accesses one after the other (48 us for the kernel at 64 rows of 64 columns; 32 now).
     // The tables come to shared memory instead, PICK_ROWS rows at a time in 16-byte loads from
     // the boundary at or before their start, and the walk costs a shared-memory access per row.
     extern __shared__ __align__(16) int16_t pick_tab[]; // up to 7 entries of the boundary, [PICK_ROWS][NS]
