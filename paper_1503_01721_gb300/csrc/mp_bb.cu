@@ -79,7 +79,6 @@ struct MPArgs {
     float *yprev;
     double *part;  // fallback solver: [P][n + 1] doubles
     double *cpart; // fallback solver: [P]
-    int32_t P;
     // exchange of the persistent solvers (see exchange_columns): tagged float pairs
     ulonglong2 *slots; // [n + 1][pstride]: column k of CTA c at k * pstride + c
     ulonglong2 *res;   // [RES_COPIES][rstride]: the reduced columns, then the elastic solver's epoch
@@ -454,7 +453,6 @@ __device__ __forceinline__ bool column_sum_cta(const ulonglong2 *col, int n_cta,
 // epoch (gctl[3]) and the set of problems still iterating (gctl[4..5]) before it
 // releases the others: the CTA split that follows reads only these words, which
 // no CTA changes until every CTA has arrived at the next batch barrier.
-struct MPArgs;
 __device__ bool batch_sync(unsigned *gctl, unsigned n_cta, const MPArgs *args, int n_plans);
 
 // Solver state every CTA keeps in shared memory (identical in all CTAs but for cta), and
@@ -504,7 +502,10 @@ struct SolveSmem {
 
 // Resident CTAs per SM the persistent solvers are compiled for (a register budget): what
 // their shared memory (solve_smem) lets an SM hold, four up to 4 apertures, two up to 44
-// (the 48 of the last kernel of that class), else one.
+// (the 48 of the last kernel of that class), else one.  At the limits of a class a few words are
+// spilled (4 bytes stored a thread; in the batched solver 8-24 for 25-64 apertures).  No aperture count from 2 to 96 is slower for it per iteration, at 12K, 180K and 1.1M voxels, than with the
+// budgets before (4, 3, 2 and 1 CTAs up to 8, 24, 48 and 96): 1.1M voxels, 8 / 24 / 48 / 64 apertures 18.4 / 23.7 /
+// 38.7 / 50.3 -> 16.9 / 21.7 / 36.0 / 47.0 us, the exchange included.
 __host__ __device__ constexpr int mp_min_ctas(int nmax) { return nmax <= 4 ? 4 : (nmax <= 48 ? 2 : 1); }
 
 // CTAs a solve of nmax apertures has at most (room for a column's staged slots; up to 160 SMs).
@@ -1317,11 +1318,12 @@ __device__ bool batch_sync(unsigned *gctl, unsigned n_cta, const MPArgs *args, i
 
 // Several independent problems in one persistent launch.  All CTAs are split
 // among the problems still iterating, in proportion to their warp tiles (the same
-// computation in every CTA); each problem has its own grid barrier.  When a
-// problem stops it bumps the batch epoch (gctl[2]); every other problem sees the
-// change at its next second barrier, saves its state and joins a barrier of the
-// whole grid (gctl[0..1]), after which the CTAs are split again among the
-// problems left.  Every problem has n apertures.
+// computation in every CTA), and each problem exchanges its sums among its own CTAs.
+// When a problem stops it bumps the batch epoch (gctl[2]); the owner of a problem's last
+// column sends the epoch along with that column's sum, so all CTAs of a problem see a
+// change at the same exchange, save its state and join a barrier of the whole grid
+// (gctl[0..1]), after which the CTAs are split again among the problems left.  Every
+// problem has n apertures.
 template <int NMAX>
 __global__ void __launch_bounds__(MP_THREADS, mp_min_ctas(NMAX))
     mp_solve_batched_kernel(const MPArgs *__restrict__ args, const int64_t *__restrict__ weight, int32_t n_plans,
@@ -2007,7 +2009,6 @@ static void mp_fill_args(MPArgs &a, void *ws, int n_cap, int p_max, const float 
     a.z = z;
     a.lo = lo;
     a.hi = hi;
-    a.P = L.P;
     a.pstride = p_max;
     a.n_tiles = (int32_t)((V + MP_THREADS - 1) / MP_THREADS);
     a.n_wtiles = ((int64_t)V + MP_WT - 1) / MP_WT;
