@@ -285,8 +285,8 @@ vmat_status dose_forward_impl(const Ddc &h, const float *x, float *d, bool compa
 // configurations that read the 16-bit index 2 plus a 4-byte base per chunk and an 8-byte chunk
 // pointer per row) once, an 8-byte row pointer per row.  Dense inputs, outputs and scales are the
 // caller's.  A pass that reads the packed stream is counted at the CSR's bytes too, the metric's
-// definition (an effective rate, not one to hold against a peak); the stream moves about 0.83 (FP32),
-// 0.78 (BF16) and 0.72 (FP8) of them at 1,300 entries per row (vmat_ddc_stream_bytes).
+// definition (an effective rate, not one to hold against a peak); the stream moves 0.82 (FP32),
+// 0.74 (BF16) and 0.67 (FP8) of them at 1,313 entries per row (vmat_ddc_stream_bytes).
 inline double csr_pass_bytes(int cfg, int vb, double nnz, double rows, double chunks) {
     if (spmv_config_index16(cfg)) return nnz * (vb + 2) + 4.0 * chunks + 16.0 * rows;
     return nnz * (vb + 4) + 8.0 * rows;
