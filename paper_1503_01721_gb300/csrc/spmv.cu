@@ -1066,33 +1066,38 @@ template <typename VT> static void pick(int cfg, bool strm, Numbering num, Launc
     else pick<ROWS_ALL, VT>(cfg, strm, n);
 }
 
+// All numberings of a configuration and form are looked up together: a caller that has run one of them
+// may capture another, whose kernel is then loaded already.
 static vmat_status launch_info(vmat_dtype dt, int cfg, bool strm, Numbering num, Launch *out) {
     static std::mutex mu;
     static Launch cache[3][N_CFG][2][N_NUMBERINGS];
-    static int cached_dev[3][N_CFG][2][N_NUMBERINGS];
+    static int cached_dev[3][N_CFG][2];
     int dev;
     VMAT_CUDA(cudaGetDevice(&dev));
     std::lock_guard<std::mutex> lock(mu);
-    Launch &L = cache[dt][cfg][strm][num];
-    if ((L.tile || L.row) && cached_dev[dt][cfg][strm][num] == dev) {
-        *out = L;
+    Launch *L = cache[dt][cfg][strm];
+    if ((L[0].tile || L[0].row) && cached_dev[dt][cfg][strm] == dev) {
+        *out = L[num];
         return VMAT_OK;
     }
-    Launch n;
-    n.threads = kCfgs[cfg].threads;
-    if (dt == VMAT_F32) pick<float>(cfg, strm, num, n);
-    else if (dt == VMAT_BF16) pick<__nv_bfloat16>(cfg, strm, num, n);
-    else pick<__nv_fp8_e4m3>(cfg, strm, num, n);
-    if (n.tile) {
-        VMAT_CUDA(cudaFuncSetAttribute(n.tile, cudaFuncAttributeMaxDynamicSharedMemorySize, n.smem));
-        VMAT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n.blocks_per_sm, n.tile, n.threads, n.smem));
-    } else {
-        VMAT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n.blocks_per_sm, n.row, n.threads, 0));
+    Launch found[N_NUMBERINGS];
+    for (int q = 0; q < N_NUMBERINGS; ++q) {
+        Launch &n = found[q];
+        n.threads = kCfgs[cfg].threads;
+        if (dt == VMAT_F32) pick<float>(cfg, strm, (Numbering)q, n);
+        else if (dt == VMAT_BF16) pick<__nv_bfloat16>(cfg, strm, (Numbering)q, n);
+        else pick<__nv_fp8_e4m3>(cfg, strm, (Numbering)q, n);
+        if (n.tile) {
+            VMAT_CUDA(cudaFuncSetAttribute(n.tile, cudaFuncAttributeMaxDynamicSharedMemorySize, n.smem));
+            VMAT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n.blocks_per_sm, n.tile, n.threads, n.smem));
+        } else {
+            VMAT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n.blocks_per_sm, n.row, n.threads, 0));
+        }
+        if (n.blocks_per_sm < 1) return set_error(VMAT_ECUDA, "spmv: configuration %d does not fit on an SM", cfg);
     }
-    if (n.blocks_per_sm < 1) return set_error(VMAT_ECUDA, "spmv: configuration %d does not fit on an SM", cfg);
-    L = n;
-    cached_dev[dt][cfg][strm][num] = dev;
-    *out = n;
+    for (int q = 0; q < N_NUMBERINGS; ++q) L[q] = found[q];
+    cached_dev[dt][cfg][strm] = dev;
+    *out = L[num];
     return VMAT_OK;
 }
 
