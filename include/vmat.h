@@ -98,9 +98,10 @@ typedef struct {
     int32_t build_Dt;   /* nonzero: build CSR(D^T), beamlet rows (beamlet_price) */
     int32_t tile_cfg;   /* SpMV configuration index of CSR(D) (and of CSR(D^T) when tile_cfg_Dt < 0),
                            -1 = library default */
-    int32_t autotune;   /* nonzero: time every tile configuration and keep the fastest.  Such a build,
+    int32_t autotune;   /* nonzero: time every configuration and keep the fastest.  Such a build,
                            and one with a consecutive-lane configuration (9-11), also holds each CSR as
-                           a packed stream that those configurations read (records of 128 entries with
+                           a packed stream that those configurations read (an autotuned one only while it
+                           is faster than the CSR: see vmat_ddc_stream_bytes; records of 128 entries with
                            16-bit column offsets: s_val + 2.1 bytes per entry, rows padded to whole
                            records; same sums, same bits), where at least half of the device's memory
                            stays free, rows are long enough to fill records and the columns of
